@@ -619,6 +619,9 @@ int hg_k_granule() { return BK; }
 int hg_tile_n(const HalfGemmDesc& d) {
     // 64-column blocks are the unit of the epilogue's bf16 stores and of an MN-major B box (one per CTA of a pair)
     const int g = (d.b_sk != 1 && cta_group(d) == 2) ? 128 : 64;
+    // The logits keep whole tiles however few patterns there are: a stored exponential is rounded to bfloat16 relative to the
+    // running maximum of its tile, so that a narrower tile gives other values (4e-4 of the gradient of 312 patterns of 128-370-2198).
+    if (d.epi == EPI_LOGITS) return (int)((d.N + g - 1) / g * g < BN_MAX ? (d.N + g - 1) / g * g : BN_MAX);
     return column_tile(d.M, d.N, d.K, d.epi, hg_tile_m(d), hg_slots(d), g, g);
 }
 
