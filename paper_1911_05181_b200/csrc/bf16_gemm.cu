@@ -265,7 +265,7 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             float run_m = -INFINITY, run_s = 0.f, zl = 0.f;
             bool have_zl = false;
             int lab = -1;
-            if (EPI == EPI_LOGITS && rv) lab = __ldg(d.labels + r);        // asked for before the wait for the products
+            if (EPI == EPI_LOGITS && rv) lab = chain_ld(d.labels + r);        // asked for before the wait for the products
             // TANH_SSE: the targets of a 64-column block are brought into L2 one block ahead of their use
             auto prefetch_targets = [&](int b64) {
                 const int c0 = n0 + b64 * 64;
@@ -308,12 +308,12 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         if (bias_vec && nvalid == 32) {
 #pragma unroll
                             for (int j = 0; j < 32; j += 4) {
-                                const float4 bb = __ldg(reinterpret_cast<const float4*>(d.bias + c0 + j));
+                                const float4 bb = chain_ld(reinterpret_cast<const float4*>(d.bias + c0 + j));
                                 bv[cc][j] = bb.x; bv[cc][j + 1] = bb.y; bv[cc][j + 2] = bb.z; bv[cc][j + 3] = bb.w;
                             }
                         } else {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) bv[cc][j] = (j < nvalid) ? __ldg(d.bias + c0 + j) : 0.f;
+                            for (int j = 0; j < 32; ++j) bv[cc][j] = (j < nvalid) ? chain_ld(d.bias + c0 + j) : 0.f;
                         }
                     }
                 }
@@ -356,9 +356,9 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 #pragma unroll
                             for (int j = 0; j < 32; j += 4) {
                                 float4 t4;
-                                if (t_vec && full) t4 = __ldg(reinterpret_cast<const float4*>(tp + j));
-                                else t4 = make_float4(j < nvalid ? __ldg(tp + j) : 0.f, j + 1 < nvalid ? __ldg(tp + j + 1) : 0.f,
-                                                      j + 2 < nvalid ? __ldg(tp + j + 2) : 0.f, j + 3 < nvalid ? __ldg(tp + j + 3) : 0.f);
+                                if (t_vec && full) t4 = chain_ld(reinterpret_cast<const float4*>(tp + j));
+                                else t4 = make_float4(j < nvalid ? chain_ld(tp + j) : 0.f, j + 1 < nvalid ? chain_ld(tp + j + 1) : 0.f,
+                                                      j + 2 < nvalid ? chain_ld(tp + j + 2) : 0.f, j + 3 < nvalid ? chain_ld(tp + j + 3) : 0.f);
                                 const float tt[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
                                 for (int t = 0; t < 4; ++t) {
@@ -407,7 +407,7 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                             if (h_vec && full) {
 #pragma unroll
                                 for (int j = 0; j < 32; j += 8) {
-                                    const uint4 w = __ldg(reinterpret_cast<const uint4*>(hp + j));
+                                    const uint4 w = chain_ld(reinterpret_cast<const uint4*>(hp + j));
                                     const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                                     for (int t = 0; t < 4; ++t) {
@@ -537,7 +537,7 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
 // dst[r][j] = bf16(src[r][j]) for j < cols; dst[r][cols] = 1 when `ones`; 0 up to the next multiple of eight.
 // One thread per 8 output elements (one 16-byte store).
-__global__ void to_bf16_kernel(const float* __restrict__ src, int64_t rows, int64_t cols, int64_t lds,
+__global__ void to_bf16_kernel(const float* src, int64_t rows, int64_t cols, int64_t lds,
                                __nv_bfloat16* __restrict__ dst, int64_t ldd, int ones) {
     chain_wait();
     const int64_t groups = (cols + (ones ? 1 : 0) + 7) >> 3;
@@ -548,11 +548,11 @@ __global__ void to_bf16_kernel(const float* __restrict__ src, int64_t rows, int6
         float v[8];
         const float* s = src + r * lds + j0;
         if (vec && j0 + 8 <= cols) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(s)), b = __ldg(reinterpret_cast<const float4*>(s) + 1);
+            const float4 a = chain_ld(reinterpret_cast<const float4*>(s)), b = chain_ld(reinterpret_cast<const float4*>(s) + 1);
             v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
         } else {
 #pragma unroll
-            for (int t = 0; t < 8; ++t) v[t] = (j0 + t < cols) ? __ldg(s + t) : ((ones && j0 + t == cols) ? 1.f : 0.f);
+            for (int t = 0; t < 8; ++t) v[t] = (j0 + t < cols) ? chain_ld(s + t) : ((ones && j0 + t == cols) ? 1.f : 0.f);
         }
         *reinterpret_cast<uint4*>(dst + r * ldd + j0) =
             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));

@@ -394,7 +394,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool c_vec = ((((uintptr_t)d.C) & 15) == 0) && ((d.ldc & 3) == 0);
         const bool t_vec = (EPI == EPI_TANH_SSE) && ((((uintptr_t)d.T) & 15) == 0) && ((d.ldt & 3) == 0);
         const bool h_vec = (EPI == EPI_TANHP) && ((((uintptr_t)d.Hm) & 15) == 0) && ((d.ldh & 3) == 0);
-        const uint32_t c_max = (EPI == EPI_BIAS_TANH && THREE_X && p.c_pair) ? __ldg(d.c_max) : 0u;
+        const uint32_t c_max = (EPI == EPI_BIAS_TANH && THREE_X && p.c_pair) ? chain_ld(d.c_max) : 0u;
         const float one = PAIR_UNIT * pair_unscale(c_max);          // what the ones column holds, before scaling
         uint32_t tile_i = 0, stg_i = 0;
         uint32_t reads[2] = {0, 0};             // how often each TMEM region has been waited for
@@ -414,7 +414,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
                 for (int j = 0; j < PER_WARP / 32; ++j) {
                     const int idx = ew * PER_WARP + j * 32 + lane;
-                    bias_s[idx] = n0 + idx < (int)d.N ? __ldg(d.bias + n0 + idx) : 0.f;
+                    bias_s[idx] = n0 + idx < (int)d.N ? chain_ld(d.bias + n0 + idx) : 0.f;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->bias_full));
@@ -452,7 +452,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             for (int c = 0; c < BN_MAX / 32; ++c) tile_max[c] = 0.f;
             int lab = -1;
             bool have_zl = false;
-            if (EPI == EPI_LOGITS && rv) lab = __ldg(d.labels + r);
+            if (EPI == EPI_LOGITS && rv) lab = chain_ld(d.labels + r);
             for (int c = 0; c < chunks; ++c) {
                 const int c0 = n0 + c * 32;
                 const int nvalid = min(32, (int)d.N - c0);      // < 32 only in the last block of a row of the matrix
@@ -505,12 +505,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             if (t_vec && full) {
 #pragma unroll
                                 for (int j = 0; j < 32; j += 4) {
-                                    const float4 q4 = __ldg(reinterpret_cast<const float4*>(tp + j));
+                                    const float4 q4 = chain_ld(reinterpret_cast<const float4*>(tp + j));
                                     t[j] = q4.x; t[j + 1] = q4.y; t[j + 2] = q4.z; t[j + 3] = q4.w;
                                 }
                             } else {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) t[j] = (j < nvalid) ? __ldg(tp + j) : 0.f;
+                                for (int j = 0; j < 32; ++j) t[j] = (j < nvalid) ? chain_ld(tp + j) : 0.f;
                             }
                         } else {
 #pragma unroll
@@ -562,14 +562,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         if (h_vec && full) {
 #pragma unroll
                             for (int j = 0; j < 32; j += 4) {
-                                const float4 h = __ldg(reinterpret_cast<const float4*>(hp + j));
+                                const float4 h = chain_ld(reinterpret_cast<const float4*>(hp + j));
                                 v[j] *= (1.f - h.x * h.x); v[j + 1] *= (1.f - h.y * h.y);
                                 v[j + 2] *= (1.f - h.z * h.z); v[j + 3] *= (1.f - h.w * h.w);
                             }
                         } else {
 #pragma unroll
                             for (int j = 0; j < 32; ++j) {
-                                if (j < nvalid) { const float h = __ldg(hp + j); v[j] = (1.f - h * h) * v[j]; } else v[j] = 0.f;
+                                if (j < nvalid) { const float h = chain_ld(hp + j); v[j] = (1.f - h * h) * v[j]; } else v[j] = 0.f;
                             }
                         }
                     } else {
@@ -717,7 +717,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
                 for (int i = 0; i < NA; ++i) {
                     const int pat = m0 + a_row + ROW_STEP * i;
-                    if (pat < n_patterns) row_lab[i] = __ldg(d.labels + pat);
+                    if (pat < n_patterns) row_lab[i] = chain_ld(d.labels + pat);
                 }
             }
             int k0 = (int)kbeg;
@@ -737,14 +737,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
                         for (int i = 0; i < NA; ++i) {
                             const int pat = m0 + a_row + ROW_STEP * i;
-                            if (pat < n_patterns && k0 < n_classes) pc_scale[i] = __ldg(d.scale + (int64_t)pat * d.scale_ld + (k0 >> 5));
+                            if (pat < n_patterns && k0 < n_classes) pc_scale[i] = chain_ld(d.scale + (int64_t)pat * d.scale_ld + (k0 >> 5));
                         }
                     } else if (kpat < n_patterns) {
-                        k_lab = __ldg(d.labels + kpat);
+                        k_lab = chain_ld(d.labels + kpat);
 #pragma unroll
                         for (int i = 0; i < NA; ++i) {
                             const int cls0 = m0 + 32 * (mn_g0 + mn_gstep * i);
-                            if (cls0 < n_classes) pc_scale[i] = __ldg(d.scale + (int64_t)kpat * d.scale_ld + (cls0 >> 5));
+                            if (cls0 < n_classes) pc_scale[i] = chain_ld(d.scale + (int64_t)kpat * d.scale_ld + (cls0 >> 5));
                         }
                     }
                 }
