@@ -940,6 +940,7 @@ int tc_tile_n(const GemmDesc& d) {
     return column_tile(d.M, d.N, d.K, d.epi, tc_tile_m(d), tc_slots(d), (b_mn && tc_cta_group(d) == 2) ? 64 : 32, 64);
 }
 
+bool tc_available() { return encode_fn() != nullptr; }
 bool tc_operand_addressable(const float* base, int64_t ld) { return encode_fn() != nullptr && operand_ok(base, ld, 0); }
 
 bool tc_gemm_supported(const GemmDesc& d) {

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_1911_05181_b200 import binding as ul, buildlib
 
@@ -177,3 +178,15 @@ def test_workspace_query_for_given_operands_is_host_only():
     assert lib.ulsnn_sgemm_workspace_bytes_for(b"N", b"N", 4, 4, 4, None, 3, None, 4, 0, ctypes.byref(out)) == ul.ERR_INVALID_ARG
     assert lib.ulsnn_sgemm_workspace_bytes_for(b"N", b"N", 4, 4, 4, None, 4, None, 4, 0, None) == ul.ERR_INVALID_ARG
     assert lib.ulsnn_sgemm_workspace_bytes_for(b"N", b"N", 4, 4, 4, None, 4, None, 4, 9, ctypes.byref(out)) == ul.ERR_INVALID_ARG
+
+
+def test_default_mode_without_a_tensor_map_encoder_is_laid_out_for_the_ffma_engine():
+    # no driver: every product of the default mode runs on the FFMA engine, which needs fp32 activations and deltas; on top of
+    # the FFMA mode's buffers there are the (hi, lo) copies of the weights, the padded batch and the fill slices of another tile size
+    if torch.cuda.is_available():
+        pytest.skip("the driver and its encoder are there")
+    sizes, n = [40, 48, 36, 20], 500
+    up = lambda x: (x + 255) // 256 * 256
+    row = lambda c: (c * 4 + (127 if c * 4 >= 512 else 31)) // (128 if c * 4 >= 512 else 32) * (128 if c * 4 >= 512 else 32)
+    copies = sum(2 * up(b * row(a)) for a, b in zip(sizes, sizes[1:])) + up(n * row(sizes[0]))
+    assert ul.mlp_workspace_bytes(sizes, ul.MATH_3XTF32, n) == ul.mlp_workspace_bytes(sizes, ul.MATH_FP32_SIMT, n) + copies
