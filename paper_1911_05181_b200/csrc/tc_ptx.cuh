@@ -352,13 +352,18 @@ inline int sm_count_of_current_device(int fallback) {
     return n;
 }
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) applies to the current device only: once per kernel and device.
-// `done` is the kernel's own bit mask over the device slots.
+// `done` is the kernel's own bit mask over the device slots.  `regs` not 0: the registers per thread that the kernel's setmaxnreg
+// shares add up to; compiled with any other number the `inc` side would wait for registers that nobody gives back, so it is not launched.
 template <class Kernel>
-inline bool allow_dynamic_smem(Kernel kernel, int bytes, std::atomic<uint64_t>& done) {
+inline bool allow_dynamic_smem(Kernel kernel, int bytes, std::atomic<uint64_t>& done, int regs = 0) {
     const int slot = current_device_slot();
     if (slot < 0) return false;
     const uint64_t bit = 1ull << slot;
     if (done.load(std::memory_order_acquire) & bit) return true;
+    if (regs != 0) {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess || fa.numRegs != regs) return false;
+    }
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
     done.fetch_or(bit, std::memory_order_release);
     return true;
