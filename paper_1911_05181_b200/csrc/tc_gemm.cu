@@ -100,6 +100,7 @@ struct Ctrl {
     volatile int abort;
     unsigned long long wait_limit;
 };
+static_assert(sizeof(Ctrl) <= COL_FACTORS_AT && COL_FACTORS_AT + 2 * BN_MAX <= CTRL_BYTES, "control page");
 
 // softmax(z) - onehot from a stored exponential e = exp(z - m) and its chunk's factor exp(m - lse); 0 outside the matrix
 __device__ __forceinline__ float delta_of(float e, float scale, int cls, int label, int n_classes) {
@@ -394,8 +395,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool c_vec = ((((uintptr_t)d.C) & 15) == 0) && ((d.ldc & 3) == 0);
         const bool t_vec = (EPI == EPI_TANH_SSE) && ((((uintptr_t)d.T) & 15) == 0) && ((d.ldt & 3) == 0);
         const bool h_vec = (EPI == EPI_TANHP) && ((((uintptr_t)d.Hm) & 15) == 0) && ((d.ldh & 3) == 0);
-        const uint32_t c_max = (EPI == EPI_BIAS_TANH && THREE_X && p.c_pair) ? chain_ld(d.c_max) : 0u;
-        const float one = PAIR_UNIT * pair_unscale(c_max);          // what the ones column holds, before scaling
+        uint16_t* factors_s = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(ctrl) + COL_FACTORS_AT);     // of the output pair's columns
         uint32_t tile_i = 0, stg_i = 0;
         uint32_t reads[2] = {0, 0};             // how often each TMEM region has been waited for
         bool ok = true;
@@ -415,6 +415,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 for (int j = 0; j < PER_WARP / 32; ++j) {
                     const int idx = ew * PER_WARP + j * 32 + lane;
                     bias_s[idx] = n0 + idx < (int)d.N ? chain_ld(d.bias + n0 + idx) : 0.f;
+                    if (EPI == EPI_BIAS_TANH && THREE_X && p.c_pair)
+                        factors_s[idx] = n0 + idx <= (int)d.N ? one_factor(pair_scale_field(chain_ld(d.c_max + n0 + idx))) : 0;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->bias_full));
@@ -625,13 +627,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         // rows are written up to their length: the ones column and zeros behind the matrix
                         if (!full) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) if (j >= nvalid) v[j] = (j == nvalid) ? one : 0.f;
+                            for (int j = 0; j < 32; ++j) if (j >= nvalid) v[j] = (j == nvalid) ? 1.f : 0.f;
+                        }
+                        const uint4* fs = reinterpret_cast<const uint4*>(factors_s + c * 32);
+#pragma unroll
+                        for (int j = 0; j < 32; j += 8) {
+                            const uint4 w4 = fs[j >> 3];
+                            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) v[j + t] *= one_of(w[t >> 1], t & 1);
                         }
                         uint8_t* blk = stg + (stg_i & 1) * EPI_STAGE_BYTES;
                         ++stg_i;
                         if (lane == 0) bulk_wait_read_1();
                         __syncwarp();
-                        stage_pair_block(blk, lane, v, pair_scale(c_max));
+                        stage_pair_block(blk, lane, v);
                         proxy_fence_async();
                         __syncwarp();
                         if (lane == 0 && r0w < d.M) {

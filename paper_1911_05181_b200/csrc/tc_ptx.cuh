@@ -313,16 +313,26 @@ __device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
 }
 
 // ------------------------------------------------------------------------------------------ fp16 pairs
-// Stages a 32 x 32 block of scale*v as an fp16 pair: 64-byte rows in 64B swizzle, the hi plane in the first 2 KB of `blk`, the
+// Exponent fields of a tile's column factors (powers of two), kept for the epilogue warps in the control page behind the barriers: 256
+// half words.  Where a column has one factor they are its bfloat16 bits; where it has two, the low byte is the exponent field of
+// the one, the high byte that of the other.  The words of two columns give the factors by a shift and a mask.
+constexpr int COL_FACTORS_AT = 512;
+__device__ __forceinline__ uint16_t one_factor(uint32_t field) { return (uint16_t)(field << 7); }
+__device__ __forceinline__ uint16_t two_factors(uint32_t f, uint32_t g) { return (uint16_t)(f | (g << 8)); }
+__device__ __forceinline__ float one_of(uint32_t w, int odd) { return __uint_as_float(odd ? w & 0xFFFF0000u : w << 16); }
+__device__ __forceinline__ float first_of(uint32_t w, int odd) { return __uint_as_float((odd ? w << 7 : w << 23) & 0x7F800000u); }
+__device__ __forceinline__ float second_of(uint32_t w, int odd) { return __uint_as_float((odd ? w >> 1 : w << 15) & 0x7F800000u); }
+
+// Stages a 32 x 32 block of scaled values as an fp16 pair: 64-byte rows in 64B swizzle, the hi plane in the first 2 KB of `blk`, the
 // lo plane in the second; this lane's row.  One TMA store of a {32, 32, 2} box writes both.
-__device__ __forceinline__ void stage_pair_block(uint8_t* blk, int lane, const float (&v)[32], float scale) {
+__device__ __forceinline__ void stage_pair_block(uint8_t* blk, int lane, const float (&v)[32]) {
     uint4* hi = reinterpret_cast<uint4*>(blk + lane * 64);
     uint4* lo = reinterpret_cast<uint4*>(blk + 2048 + lane * 64);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         uint32_t h[4], l[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) split_pair(v[8 * j + 2 * t] * scale, v[8 * j + 2 * t + 1] * scale, h[t], l[t]);
+        for (int t = 0; t < 4; ++t) split_pair(v[8 * j + 2 * t], v[8 * j + 2 * t + 1], h[t], l[t]);
         hi[j ^ ((lane >> 1) & 3)] = make_uint4(h[0], h[1], h[2], h[3]);
         lo[j ^ ((lane >> 1) & 3)] = make_uint4(l[0], l[1], l[2], l[3]);
     }
