@@ -80,3 +80,28 @@ def test_a_tiny_unit_between_two_hidden_layers(factor):
     Ws[0][9] *= f; bs[0][9] *= f            # layer 1
     X, y = si.mlp_batch(52, sizes, n)
     _check(Ws, bs, X, labels=y)
+
+
+# One target far above the others: the other patterns keep their deltas and the other classes their rows.  The pattern's first
+# inputs are zero, so that the gradient's columns there do not see it at all.
+@pytest.mark.parametrize("sizes", [[40, 48, 20], [40, 48, 36, 20], [40, 48, 36, 1100]])
+@pytest.mark.parametrize("target", [1e6, 1e8, 1e10, 1e12, 1e15])
+def test_a_target_far_above_the_others(target, sizes):
+    n = 150
+    Ws, bs = _net(53, sizes)
+    X, _ = si.mlp_batch(53, sizes, n)
+    X[7, :10] = 0
+    T = si.mlp_targets(53, sizes, n, 0, False)
+    T[7, 2] = np.float32(target)
+    _check(Ws, bs, X, T=T)
+
+
+# Output units whose deltas are all small (targets reached to 2^-20), and a hidden layer whose outgoing weights differ
+@pytest.mark.parametrize("scale", [2.0 ** -16, 2.0 ** -30])
+def test_classes_and_hidden_units_with_small_deltas(scale):
+    sizes, n = [40, 48, 36, 20], 300
+    Ws, bs = _net(54, sizes)
+    X, _ = si.mlp_batch(54, sizes, n)
+    Ws[2][:, 5] *= np.float32(scale)            # deltas of unit 5 of layer 2
+    T = si.mlp_targets(54, sizes, n, 0, False)
+    _check(Ws, bs, X, T=T)
