@@ -105,3 +105,15 @@ def test_classes_and_hidden_units_with_small_deltas(scale):
     Ws[2][:, 5] *= np.float32(scale)            # deltas of unit 5 of layer 2
     T = si.mlp_targets(54, sizes, n, 0, False)
     _check(Ws, bs, X, T=T)
+
+
+# Classes that the softmax hardly ever predicts and that are nobody's label: their rows are sums of tiny probabilities
+@pytest.mark.parametrize("sizes,n", [([40, 48, 24], 200), ([40, 48, 36, 24], 200), ([24, 40, 12300], 40), ([40, 64, 1100], 700)])
+@pytest.mark.parametrize("log10_p", [-5, -9, -11, -13, -25])
+def test_classes_that_are_hardly_ever_predicted(sizes, n, log10_p):
+    Ws, bs = _net(55, sizes)
+    rare = np.arange(1, sizes[-1], 5)
+    bs[-1][rare] += np.float32(log10_p * np.log(10.0))
+    X, y = si.mlp_batch(55, sizes, n)
+    y = np.where(np.isin(y, rare), 0, y).astype(np.int32)
+    _check(Ws, bs, X, labels=y)
