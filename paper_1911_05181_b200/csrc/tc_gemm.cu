@@ -765,56 +765,45 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 float4* a_lo = reinterpret_cast<float4*>(base + off_a_lo);
                 float4* b_hi = reinterpret_cast<float4*>(base + off_b_hi);
                 float4* b_lo = reinterpret_cast<float4*>(base + off_b_lo);
-                // The body is instantiated per mode so that its unrolled loops are straight-line code.
-                auto pass = [&](auto three_tag) {
-                    constexpr bool THREE = decltype(three_tag)::value;
-                    {
-                    float4 x[NA];
+                float4 x[NA];
 #pragma unroll
-                    for (int i = 0; i < NA; ++i) x[i] = a_hi[st + NT * i];
-                    if (d.a_transform) {
-                        if (!p.a_mn) {
-                            const int cls = k0 + kch * 4;
+                for (int i = 0; i < NA; ++i) x[i] = a_hi[st + NT * i];
+                if (d.a_transform) {
+                    if (!p.a_mn) {
+                        const int cls = k0 + kch * 4;
 #pragma unroll
-                            for (int i = 0; i < NA; ++i) {
-                                const bool live = m0 + a_row + ROW_STEP * i < n_patterns;
-                                x[i].x = live ? delta_of(x[i].x, pc_scale[i], cls + 0, row_lab[i], n_classes) : 0.f;
-                                x[i].y = live ? delta_of(x[i].y, pc_scale[i], cls + 1, row_lab[i], n_classes) : 0.f;
-                                x[i].z = live ? delta_of(x[i].z, pc_scale[i], cls + 2, row_lab[i], n_classes) : 0.f;
-                                x[i].w = live ? delta_of(x[i].w, pc_scale[i], cls + 3, row_lab[i], n_classes) : 0.f;
-                            }
-                        } else {
-                            const bool live = kpat < n_patterns;
+                        for (int i = 0; i < NA; ++i) {
+                            const bool live = m0 + a_row + ROW_STEP * i < n_patterns;
+                            x[i].x = live ? delta_of(x[i].x, pc_scale[i], cls + 0, row_lab[i], n_classes) : 0.f;
+                            x[i].y = live ? delta_of(x[i].y, pc_scale[i], cls + 1, row_lab[i], n_classes) : 0.f;
+                            x[i].z = live ? delta_of(x[i].z, pc_scale[i], cls + 2, row_lab[i], n_classes) : 0.f;
+                            x[i].w = live ? delta_of(x[i].w, pc_scale[i], cls + 3, row_lab[i], n_classes) : 0.f;
+                        }
+                    } else {
+                        const bool live = kpat < n_patterns;
 #pragma unroll
-                            for (int i = 0; i < NA; ++i) {
-                                const int cls = m0 + 32 * (mn_g0 + mn_gstep * i) + mch * 4;
-                                x[i].x = live ? delta_of(x[i].x, pc_scale[i], cls + 0, k_lab, n_classes) : 0.f;
-                                x[i].y = live ? delta_of(x[i].y, pc_scale[i], cls + 1, k_lab, n_classes) : 0.f;
-                                x[i].z = live ? delta_of(x[i].z, pc_scale[i], cls + 2, k_lab, n_classes) : 0.f;
-                                x[i].w = live ? delta_of(x[i].w, pc_scale[i], cls + 3, k_lab, n_classes) : 0.f;
-                            }
+                        for (int i = 0; i < NA; ++i) {
+                            const int cls = m0 + 32 * (mn_g0 + mn_gstep * i) + mch * 4;
+                            x[i].x = live ? delta_of(x[i].x, pc_scale[i], cls + 0, k_lab, n_classes) : 0.f;
+                            x[i].y = live ? delta_of(x[i].y, pc_scale[i], cls + 1, k_lab, n_classes) : 0.f;
+                            x[i].z = live ? delta_of(x[i].z, pc_scale[i], cls + 2, k_lab, n_classes) : 0.f;
+                            x[i].w = live ? delta_of(x[i].w, pc_scale[i], cls + 3, k_lab, n_classes) : 0.f;
                         }
                     }
+                }
 #pragma unroll
-                    for (int i = 0; i < NA; ++i) {
-                        if constexpr (THREE) {
-                            float4 h, l; split4(x[i], h, l);
-                            a_hi[st + NT * i] = h; a_lo[st + NT * i] = l;
-                        } else {
-                            a_hi[st + NT * i] = x[i];       // only reached when A was transformed
-                        }
-                    }
-                    }
-                    if (THREE && !p.b_pre) {
-                        const int nvec = b_cols * CPR;               // BK*4 bytes per column of the tile
+                for (int i = 0; i < NA; ++i) {
+                    float4 h, l; split4(x[i], h, l);
+                    a_hi[st + NT * i] = h; a_lo[st + NT * i] = l;
+                }
+                if (!p.b_pre) {
+                    const int nvec = b_cols * CPR;               // BK*4 bytes per column of the tile
 #pragma unroll 4
-                        for (int idx = st; idx < nvec; idx += NT) {
-                            float4 h, l; split4(b_hi[idx], h, l);
-                            b_hi[idx] = h; b_lo[idx] = l;
-                        }
+                    for (int idx = st; idx < nvec; idx += NT) {
+                        float4 h, l; split4(b_hi[idx], h, l);
+                        b_hi[idx] = h; b_lo[idx] = l;
                     }
-                };
-                pass(std::integral_constant<bool, THREE_X>{});
+                }
                 proxy_fence_async();            // make these generic-proxy writes visible to the tensor core's reads
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->ready[s]));
