@@ -43,7 +43,10 @@ typedef int ulsnn_status_t;
 
 /* How products of fp32 numbers are formed.  Accumulation is fp32 in all modes. */
 typedef enum {
-    ULSNN_MATH_3XTF32    = 0,  /* tensor cores, each operand split hi+lo (TF32, or scaled fp16 inside a network), three products: fp32-level accuracy */
+    ULSNN_MATH_3XTF32    = 0,  /* tensor cores, each operand split hi+lo, three products: fp32-level accuracy.  TF32 parts keep 22 bits of
+                                  any value.  Inside a network the parts are scaled fp16, with scales per unit, class, pattern or row of
+                                  the weights: what is below 2^-27 of the largest value (activations: of its bound) in the same row or column
+                                  is dropped */
     ULSNN_MATH_TF32      = 1,  /* tensor cores, operands truncated to TF32 (10-bit mantissa): fast mode */
     ULSNN_MATH_FP32_SIMT = 2,  /* FFMA on the CUDA cores: exact fp32 products, the comparison kernel */
     ULSNN_MATH_BF16      = 3   /* tensor cores, operands and stored activations / deltas rounded to bfloat16 (8-bit

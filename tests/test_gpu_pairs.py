@@ -7,7 +7,7 @@ import torch
 import oracle
 import synth_inputs as si
 from paper_1911_05181_b200 import binding as ul
-from helpers import GpuNet, dev, tolerance_at
+from helpers import TOL, GpuNet, dev, tolerance_at
 
 pytestmark = pytest.mark.gpu
 
@@ -40,8 +40,8 @@ def test_tile_and_stage_edges(sizes, n):
     _check(sizes, n, Ws, bs, 41)
 
 
-# The pair's scale follows the largest weight: matrices of very small and large weights, one row a thousand times smaller than
-# the rest (its products keep their relative accuracy in the sums they are part of), and a single large weight.
+# The pairs' scales follow the largest weights: matrices of very small and large weights, one row a thousand times smaller than
+# the rest, and a single large weight.  Whole tensors are compared here; test_gpu_pair_ranges.py looks at rows and columns.
 @pytest.mark.parametrize("form", ["small", "large", "row", "outlier"])
 def test_weight_scales(form):
     sizes, n = [40, 48, 36, 20], 200
@@ -62,6 +62,7 @@ def test_small_products_use_narrow_tiles_and_slices(math_mode, sizes, n):
     g = GpuNet(sizes, math_mode, n); g.set_params(Ws, bs)
     loss, dW, db = g.gradient(X, y)
     want, cond = oracle.mlp_gradient(Ws, bs, X, y), oracle.gradient_condition(Ws, bs, X, labels=y)
+    assert abs(loss - want[0]) <= TOL[math_mode] * abs(want[0])
     for got, ref, c in zip(dW + db, list(want[1]) + list(want[2]), list(cond[0]) + list(cond[1])):
         assert oracle.rel_l2(got, ref) <= tolerance_at(math_mode, c, "softmax"), (sizes, n)
 
