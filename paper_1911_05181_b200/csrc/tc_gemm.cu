@@ -171,7 +171,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if constexpr (CG == 2) cluster_sync_all(); else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
-    chain_wait();
+    chain_wait_only();
 
     // offsets inside a stage: the landed A and B tiles, then (3xTF32) their lo parts
     const int off_a_hi = 0, off_b_hi = A_TILE_BYTES;
@@ -812,6 +812,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
 
     // ---------------------------------------------------------------------- teardown
+    chain_release();
     if (ctrl->abort) {
         // give copies that may still be in flight time to land before the shared memory is released
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
