@@ -148,11 +148,3 @@ def test_operands_tma_cannot_address_are_rebuffered_onto_the_tensor_cores(math):
             torch.cuda.synchronize()
             assert ul.launch_counts()["tc_gemm"] > c0["tc_gemm"]
             assert oracle.rel_l2(dC.cpu().numpy(), want) <= TOL[math]
-
-
-@pytest.mark.parametrize("math,shape,slices", [(ul.MATH_3XTF32, (480, 3204, 65536), 16), (ul.MATH_3XTF32, (4096, 4096, 65536), 16), (ul.MATH_TF32, (96, 200, 20000), 37)])
-def test_an_sgemm_has_as_many_slices_as_its_longest_sums_and_the_gpu_ask_for(math, shape, slices):
-    # slices of at most 4,096 k once K is large, or two tiles per slot (but slices of 512 k) where tiles are few
-    M, N, K = shape
-    A = torch.empty(64, device="cuda")          # for its alignment only
-    assert ul.sgemm_workspace_bytes_for("T", "N", M, N, K, A, M, A, N, math) == (slices * M * N * 4 + 255) // 256 * 256
