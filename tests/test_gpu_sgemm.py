@@ -148,3 +148,11 @@ def test_operands_tma_cannot_address_are_rebuffered_onto_the_tensor_cores(math):
             torch.cuda.synchronize()
             assert ul.launch_counts()["tc_gemm"] > c0["tc_gemm"]
             assert oracle.rel_l2(dC.cpu().numpy(), want) <= TOL[math]
+
+
+@pytest.mark.parametrize("shape,slices", [((480, 3204, 65536), 17), ((96, 200, 20000), 37)])
+def test_an_sgemm_asks_for_the_scratch_of_its_slices(shape, slices):
+    # above the 8 MB of the entry point without a workspace by estimated time, below it by the rule that fills the GPU
+    M, N, K = shape
+    A = torch.empty(64, device="cuda")          # for its alignment only
+    assert ul.sgemm_workspace_bytes_for("T", "N", M, N, K, A, M, A, N, ul.MATH_3XTF32) == (slices * M * N * 4 + 255) // 256 * 256
