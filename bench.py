@@ -47,21 +47,20 @@ CHUNK = {"config4": 131072}
 MATH = {"3xtf32": 0, "tf32": 1, "simt": 2, "bf16": 3}
 NOMINAL_TF32_OVER_BF16 = 0.5        # dense TF32 tensor rate is half the BF16 rate
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture) of the products that can be the
-# dominant kernel, captured on a smaller batch and scaled by the pattern count, to which these products' traffic is
-# proportional.  Reported only while the library still is the version the counters were taken on; null otherwise.
+# dominant kernel, captured on 16384 patterns (x4), in 16-bit mode on 32768 (x2), and scaled by the pattern count, to which these products'
+# traffic is proportional but for the slices' partial products (a few per cent).  Reported only while the library still is the
+# version the counters were taken on; null otherwise.
 NCU_TRAFFIC = {
-    "library_version": 110,
-    # captured at 16384 patterns (x4); in 16-bit mode at 32768 patterns (x2)
-    # captured at 18944 patterns (x65536/18944)
-    ("config3", "3xtf32", (3203, 481, 65536)): 65536 / 18944 * (293.22470e6 + 23.882496e6),
-    ("config3", "3xtf32", (65536, 480, 3203)): 65536 / 18944 * (305.16045e6 + 27.308544e6),
-    ("config3", "3xtf32", (65536, 3203, 480)): 65536 / 18944 * (46.723840e6 + 203.48826e6),
-    ("config3", "tf32", (65536, 3203, 480)): 4 * (39.002112e6 + 162.37900e6),
-    ("config3", "tf32", (65536, 480, 3203)): 4 * (256.99609e6 + 22.658560e6),
-    ("config3", "tf32", (3203, 481, 65536)): 4 * (250.86515e6 + 21.920000e6),
-    ("config3", "bf16", (65536, 3203, 480)): 2 * (38.447872e6 + 175.91628e6),
-    ("config3", "bf16", (65536, 480, 3203)): 2 * (249.72902e6 + 20.953344e6),
-    ("config3", "bf16", (3203, 481, 65536)): 2 * (253.34092e6 + 21.497088e6),
+    "library_version": 111,
+    ("config3", "3xtf32", (65536, 3203, 480)): 4 * (41.396480e6 + 159.556864e6),
+    ("config3", "3xtf32", (65536, 480, 3203)): 4 * (280.179456e6 + 24.333824e6),
+    ("config3", "3xtf32", (3203, 481, 65536)): 4 * (255.164928e6 + 17.678336e6),
+    ("config3", "tf32", (65536, 3203, 480)): 4 * (40.698880e6 + 157.150720e6),
+    ("config3", "tf32", (65536, 480, 3203)): 4 * (256.758528e6 + 18.550016e6),
+    ("config3", "tf32", (3203, 481, 65536)): 4 * (253.641984e6 + 32.606720e6),
+    ("config3", "bf16", (65536, 3203, 480)): 2 * (39.448832e6 + 168.657152e6),
+    ("config3", "bf16", (65536, 480, 3203)): 2 * (256.808704e6 + 18.214400e6),
+    ("config3", "bf16", (3203, 481, 65536)): 2 * (256.340992e6 + 31.413504e6),
 }
 # cuBLAS through torch.matmul, 8192^3, on this machine's B200s (`--workload peaks`): TF32 allowed, best of 10 isolated
 # calls and 4 s back to back under the power cap (SM clock 1042 MHz of 1965).  Printed beside the peak the fractions use.
@@ -609,19 +608,16 @@ def main():
             mult = 3.0 if args.math == "3xtf32" else 1.0
             esize = 2.0 if half else 4.0
             achieved = mult * logical / (ms_k * 1e-3) / 1e12
-            # What the product must move, as the path lays its operands out: both operands once, the output once
-            # (split-K partials for a weight-gradient product, whose K is the pattern count), and for a delta product
-            # (phases L .. 2L-2) the hidden activations its tanh' epilogue reads; an fp16 pair is four bytes per element,
-            # like a float.
+            # What the product must move, as the path lays its operands out: both operands once, the output once, and for a
+            # delta product (phases L .. 2L-2) the hidden activations its tanh' epilogue reads; an fp16 pair is four bytes per
+            # element, like a float.
             is_delta = L <= dom < 2 * L - 1
-            is_wgrad = dom >= 2 * L - 1
             if dom < L:                 # forward: A = batch or activations, B = weights
                 alg = esize * (M * K + K * N + M * N)
             elif is_delta:              # A = output deltas / deltas, B = weights, epilogue reads H, writes delta
                 alg = esize * (M * K + K * N + M * N + M * N)
-            else:                       # A = deltas, B = activations or the batch; output: the slices' partial products
-                splits = max(1, -(-K // 4096)) if not half else max(1, -(-K // 8192))
-                alg = esize * (M * K + K * N) + 4.0 * M * N * splits
+            else:                       # A = deltas, B = activations or the batch; output in fp32, once however many slices there are
+                alg = esize * (M * K + K * N) + 4.0 * M * N
             # networks with hidden layers in 3xTF32 mode: all products but the first and the last are fp16 pairs
             on_pairs = args.math == "3xtf32" and L >= 2 and 0 < dom < 3 * L - 2
             rate = "bf16" if half or on_pairs else "tf32"

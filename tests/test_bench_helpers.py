@@ -42,3 +42,14 @@ def test_scaling_workloads_of_the_processor_scaling_experiment():
     # every shape of the SGEMM sweep with 3203 columns is there as the configuration states it (not a stand-in)
     assert ("N", "N", 65536, 3203, 480) in bench.SGEMM_SWEEP and ("T", "N", 480, 3203, 65536) in bench.SGEMM_SWEEP
     assert not any(n == 3204 for _, _, _, n, _ in bench.SGEMM_SWEEP)
+
+
+def test_traffic_counters_belong_to_the_version_they_name():
+    # counters are printed for one library version only; each table row is a product of the default workload
+    sizes, n, _ = bench.WORKLOADS["config3"]
+    products = {(n, sizes[2], sizes[1]), (n, sizes[1], sizes[2]), (sizes[2], sizes[1] + 1, n)}
+    rows = [k for k in bench.NCU_TRAFFIC if k != "library_version"]
+    assert {(m, k) for _, m, k in rows} == {(m, k) for m in ("3xtf32", "tf32", "bf16") for k in products}
+    # no row is below what the product has to read and write of its larger operand
+    for (_, m, (M, N, K)), v in ((k, bench.NCU_TRAFFIC[k]) for k in rows):
+        assert v > (2 if m == "bf16" else 4) * 0.8 * max(M * K, M * N, K * N)

@@ -110,7 +110,7 @@ def test_classes_and_hidden_units_with_small_deltas(scale):
 # Classes that the softmax hardly ever predicts and that are nobody's label: their rows are sums of tiny probabilities
 # (few and many patterns: the classes are looked for in one launch or in one of their own)
 @pytest.mark.parametrize("sizes,n", [([40, 48, 24], 200), ([40, 48, 36, 24], 200), ([24, 40, 12300], 40), ([24, 40, 12300], 180), ([40, 64, 1100], 700),
-                                     ([12, 20, 43], 4100)])
+                                     ([12, 20, 43], 4100), ([12, 16, 65600], 40)])
 @pytest.mark.parametrize("log10_p", [-5, -9, -11, -13, -25])
 def test_classes_that_are_hardly_ever_predicted(sizes, n, log10_p):
     Ws, bs = _net(55, sizes)
