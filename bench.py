@@ -48,8 +48,8 @@ MATH = {"3xtf32": 0, "tf32": 1, "simt": 2, "bf16": 3}
 NOMINAL_TF32_OVER_BF16 = 0.5        # dense TF32 tensor rate is half the BF16 rate
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture) of the products that can be the
 # dominant kernel, captured on 16384 patterns (x4), in 16-bit mode on 32768 (x2), and scaled by the pattern count, to which these products'
-# traffic is proportional but for the slices' partial products (a few per cent).  Reported only while the library still is the
-# version the counters were taken on; null otherwise.
+# traffic is proportional but for the slices' partial products (a few per cent).  Softmax head; reported only while the library still is
+# the version the counters were taken on; null otherwise.
 NCU_TRAFFIC = {
     "library_version": 111,
     ("config3", "3xtf32", (65536, 3203, 480)): 4 * (41.396480e6 + 159.556864e6),
@@ -625,7 +625,7 @@ def main():
             roofline.update(fractions(achieved, tensor_peaks(peaks, rate == "bf16"), region_ms, sm_mhz))
             roofline.update({
                 "traffic": (NCU_TRAFFIC.get((args.workload, args.math, (M, N, K)))
-                            if ul.version() == NCU_TRAFFIC["library_version"] and args.patterns <= 0 else None),
+                            if ul.version() == NCU_TRAFFIC["library_version"] and args.patterns <= 0 and args.head == "softmax" else None),
                 "algorithmic_bytes": alg,
                 "kernel": "%s M=%d N=%d K=%d" % ("bf16_gemm" if half else "pair_gemm" if on_pairs else "tc_gemm", M, N, K), "ms": ms_k,
                 "flops_counted": "%gx 2MNK" % mult, "logical_tflops": logical / (ms_k * 1e-3) / 1e12,
