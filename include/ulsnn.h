@@ -44,7 +44,8 @@ typedef int ulsnn_status_t;
 /* How products of fp32 numbers are formed.  Accumulation is fp32 in all modes. */
 typedef enum {
     ULSNN_MATH_3XTF32    = 0,  /* tensor cores, each operand split hi+lo, three products: fp32-level accuracy.  TF32 parts keep 22 bits of
-                                  any value.  Inside a network the parts are scaled fp16, with scales per unit, class, pattern or row of
+                                  any value.  Large products of ulsnn_sgemm_ex use scaled fp16 parts where a test of the operands shows
+                                  that the sums lose no more by them.  Inside a network the parts are scaled fp16, with scales per unit, class, pattern or row of
                                   the weights: what is below 2^-27 of the largest value (activations: of its bound) in the same row or column
                                   is dropped */
     ULSNN_MATH_TF32      = 1,  /* tensor cores, operands truncated to TF32 (10-bit mantissa): fast mode */
@@ -83,6 +84,12 @@ int ulsnn_version(void);
  * which is not, covers addressable operands only.  ulsnn_sgemm_ex takes the re-buffered route when the workspace it is
  * given is large enough for it and computes such a product with the FFMA kernel (at least as accurate, several times
  * slower) when it is not; C may have any alignment and ldc on either route.
+ * ULSNN_MATH_3XTF32, large products: ulsnn_sgemm_workspace_bytes_for also includes the room for both operands as pairs of scaled fp16
+ * values (as much as the operands themselves; left out where that is more than 640 MiB beyond what the product needs otherwise).  Given
+ * that much, ulsnn_sgemm_ex converts them and, on the device, looks whether the pairs hold them: no value that is not finite, and so few
+ * values below about 2^-15 of the largest in their row of op(A) or column of op(B) that what these lose is below 2^-22 of the sum of the
+ * magnitudes of any entry's terms.  If so the products run on the pairs, 1.2 to 1.8 times as fast in all; if not, on TF32
+ * parts as with less workspace, with the same result and 5 to 15 % later (values of very different size along a sum, sums of mostly zeros).
  * ulsnn_sgemm's own scratch is shared by all its calls on a device: calls on one device must be ordered with respect
  * to each other (one stream, or events), and any call that needs more scratch than every earlier one may synchronise.
  * ULSNN_MATH_BF16: op(A) and op(B) are first rounded to bfloat16 (round to nearest even) into the workspace, which

@@ -14,7 +14,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libulsnn.so")
-SOURCES = ["api.cu", "simt_gemm.cu", "tc_gemm.cu", "bf16_gemm.cu", "pair_gemm.cu", "reduce.cu"]
+SOURCES = ["api.cu", "simt_gemm.cu", "tc_gemm.cu", "bf16_gemm.cu", "pair_gemm.cu", "operand_pairs.cu", "reduce.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "tc_ptx.cuh"), os.path.join(HERE, "..", "include", "ulsnn.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]

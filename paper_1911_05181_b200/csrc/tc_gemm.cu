@@ -172,6 +172,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     chain_wait_only();
+    int units = p.units;
+    if (THREE_X && (EPI == EPI_SGEMM || EPI == EPI_PARTIAL) && d.unless && chain_ld(d.unless) != 0u) units = 0;
 
     // offsets inside a stage: the landed A and B tiles, then (3xTF32) their lo parts
     const int off_a_hi = 0, off_b_hi = A_TILE_BYTES;
@@ -182,7 +184,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // one warp fetches everything; the extra polling warps cost such products 3-5 %)
         RingPos rp{0, 0};
         bool ok = true;
-        for (int u = first_unit; u < p.units && ok; u += unit_step) {
+        for (int u = first_unit; u < units && ok; u += unit_step) {
             int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
             int64_t kbeg; int nkb, tail; unit_k_range<BK, UMMA_K>(p, sp, kbeg, nkb, tail);
             // this CTA's rows of A and its share of the tile's columns of B
@@ -237,7 +239,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool get_a = warp == 0;
         RingPos rp{0, 0};
         bool ok = true;
-        for (int u = first_unit; u < p.units && ok; u += unit_step) {
+        for (int u = first_unit; u < units && ok; u += unit_step) {
             int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
             int64_t kbeg; int nkb, tail; unit_k_range<BK, UMMA_K>(p, sp, kbeg, nkb, tail);
             // this CTA's rows of A and its share of the tile's columns of B
@@ -309,7 +311,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             uint32_t tile_i = 0;
             uint32_t overwrites[2] = {0, 0};        // how often each TMEM region has been restarted
             bool ok = true;
-            for (int u = first_unit; u < p.units && ok; u += unit_step, ++tile_i) {
+            for (int u = first_unit; u < units && ok; u += unit_step, ++tile_i) {
                 int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
                 int64_t kbeg; int nkb, tail; unit_k_range<BK, UMMA_K>(p, sp, kbeg, nkb, tail);
                 const uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(p, nt) >> 3) << 17);
@@ -369,7 +371,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             // CTA 1 issues nothing: this warp tells CTA 0 when a stage of CTA 1 is ready for the products
             RingPos rp{0, 0};
             bool ok = true;
-            for (int u = first_unit; u < p.units && ok; u += unit_step) {
+            for (int u = first_unit; u < units && ok; u += unit_step) {
                 int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
                 int64_t kbeg; int nkb, tail; unit_k_range<BK, UMMA_K>(p, sp, kbeg, nkb, tail);
                 for (int kb = 0; kb < nkb; ++kb) {
@@ -399,7 +401,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t tile_i = 0, stg_i = 0;
         uint32_t reads[2] = {0, 0};             // how often each TMEM region has been waited for
         bool ok = true;
-        for (int u = first_unit; u < p.units && ok; u += unit_step, ++tile_i) {
+        for (int u = first_unit; u < units && ok; u += unit_step, ++tile_i) {
             int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
             int64_t kbeg_; int nkb_, tail_; unit_k_range<BK, UMMA_K>(p, sp, kbeg_, nkb_, tail_);
             const int n_chunks = (nkb_ + p.chunk_blocks - 1) / p.chunk_blocks;
@@ -713,7 +715,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int n_classes = (int)p.n_classes, n_patterns = (int)p.n_patterns;
         RingPos rp{0, 0};
         bool ok = true;
-        for (int u = first_unit; u < p.units && ok; u += unit_step) {
+        for (int u = first_unit; u < units && ok; u += unit_step) {
             int mt, nt, sp; unit_coords(p, u, mt, nt, sp);
             int64_t kbeg; int nkb, tail; unit_k_range<BK, UMMA_K>(p, sp, kbeg, nkb, tail);
             const int m0 = (mt * CG + rank) * BM;
