@@ -536,26 +536,27 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
 // ------------------------------------------------------------------------------------------------ small kernels
 
-// dst[r][j] = bf16(src[r][j]) for j < cols; dst[r][cols] = 1 when `ones`; 0 up to the next multiple of eight.
-// One thread per 8 output elements (one 16-byte store).
-__global__ void to_bf16_kernel(const float* src, int64_t rows, int64_t cols, int64_t lds,
-                               __nv_bfloat16* __restrict__ dst, int64_t ldd, int ones) {
+// See ToBf16.  One thread per 8 output elements (one 16-byte store).
+__global__ void __launch_bounds__(256) to_bf16_kernel(const ToBf16 t) {
     chain_wait();
-    const int64_t groups = (cols + (ones ? 1 : 0) + 7) >> 3;
-    const int64_t total = rows * groups;
-    const bool vec = ((((uintptr_t)src) & 15) == 0) && ((lds & 3) == 0);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    int block = blockIdx.x, i = 0;
+    for (; i + 1 < t.count && block >= t.m[i].blocks; ++i) block -= t.m[i].blocks;
+    const ToBf16::Matrix& m = t.m[i];
+    const int64_t cols = m.cols, groups = (cols + (m.ones ? 1 : 0) + 7) >> 3;
+    const int64_t total = m.rows * groups;
+    const bool vec = ((((uintptr_t)m.src) & 15) == 0) && ((m.lds & 3) == 0);
+    for (int64_t e = (int64_t)block * 256 + threadIdx.x; e < total; e += (int64_t)m.blocks * 256) {
         const int64_t r = e / groups, j0 = (e - r * groups) << 3;
         float v[8];
-        const float* s = src + r * lds + j0;
+        const float* s = m.src + r * m.lds + j0;
         if (vec && j0 + 8 <= cols) {
             const float4 a = chain_ld(reinterpret_cast<const float4*>(s)), b = chain_ld(reinterpret_cast<const float4*>(s) + 1);
             v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
         } else {
 #pragma unroll
-            for (int t = 0; t < 8; ++t) v[t] = (j0 + t < cols) ? chain_ld(s + t) : ((ones && j0 + t == cols) ? 1.f : 0.f);
+            for (int k = 0; k < 8; ++k) v[k] = (j0 + k < cols) ? chain_ld(s + k) : ((m.ones && j0 + k == cols) ? 1.f : 0.f);
         }
-        *reinterpret_cast<uint4*>(dst + r * ldd + j0) =
+        *reinterpret_cast<uint4*>(m.dst + r * m.ldd + j0) =
             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
     }
 }
@@ -697,14 +698,20 @@ ulsnn_status_t hg_gemm_launch(const HalfGemmDesc& d, cudaStream_t stream) {
     return ULSNN_ERR_INVALID_ARG;
 }
 
-ulsnn_status_t launch_to_bf16(const float* src, int64_t rows, int64_t cols, int64_t lds, __nv_bfloat16* dst, int64_t ldd,
-                              int ones, cudaStream_t stream) {
-    if (rows <= 0 || cols <= 0) return ULSNN_OK;
-    if ((ldd & 7) != 0 || ldd < cols + (ones ? 1 : 0) || (((uintptr_t)dst) & 15) != 0) return ULSNN_ERR_INVALID_ARG;
-    const int64_t total = rows * ((cols + (ones ? 1 : 0) + 7) >> 3);
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 148 * 32) blocks = 148 * 32;
-    launch_chained(to_bf16_kernel, (unsigned)blocks, 256, stream, src, rows, cols, lds, dst, ldd, ones);
+ulsnn_status_t launch_to_bf16(const ToBf16& t, cudaStream_t stream) {
+    ToBf16 q{};
+    int64_t all = 0;
+    for (int i = 0; i < t.count; ++i) {
+        if (t.m[i].rows <= 0 || t.m[i].cols <= 0) continue;
+        if (t.m[i].ldd % 8 != 0 || t.m[i].ldd < t.m[i].cols + (t.m[i].ones ? 1 : 0) || (((uintptr_t)t.m[i].dst) & 15) != 0) return ULSNN_ERR_INVALID_ARG;
+        ToBf16::Matrix& m = q.m[q.count++] = t.m[i];
+        int64_t blocks = (m.rows * ((m.cols + (m.ones ? 1 : 0) + 7) >> 3) + 255) / 256;
+        if (blocks > 148 * 32) blocks = 148 * 32;
+        m.blocks = (int)blocks;
+        all += blocks;
+    }
+    if (q.count == 0) return ULSNN_OK;
+    launch_chained(to_bf16_kernel, (unsigned)all, 256, stream, q);
     count_launch(2);
     return cuda_ok(cudaGetLastError());
 }
