@@ -619,6 +619,7 @@ int hg_slots(const HalfGemmDesc& d) { return NUM_SMS / cta_group(d); }
 int hg_k_granule() { return BK; }
 
 int hg_tile_n(const HalfGemmDesc& d) {
+    if (d.tile_n) return d.tile_n;
     // 64-column blocks are the unit of the epilogue's bf16 stores and of an MN-major B box (one per CTA of a pair)
     const int g = (d.b_sk != 1 && cta_group(d) == 2) ? 128 : 64;
     // The logits keep whole tiles however few patterns there are: a stored exponential is rounded to bfloat16 relative to the

@@ -929,12 +929,13 @@ ulsnn_status_t launch_mode(bool three_x, int cg, const Maps& m, const TcParams& 
 
 // Products with more than one 128-row tile are computed by pairs of CTAs (256-row tiles, tcgen05 cta_group::2):
 // per product instruction each SM then reads half as much of B from its shared memory.
-int tc_cta_group(const GemmDesc& d) { return d.M > BM ? 2 : 1; }
+int tc_cta_group(const GemmDesc& d) { return cta_pairs(d.M, d.N, d.epi) ? 2 : 1; }
 int tc_tile_m(const GemmDesc& d) { return BM * tc_cta_group(d); }
 int tc_slots(const GemmDesc& d) { return NUM_SMS / tc_cta_group(d); }
 int tc_colsum_groups() { return 4; }
 
 int tc_tile_n(const GemmDesc& d) {
+    if (d.tile_n) return d.tile_n;
     // 32-column blocks are the unit of the epilogue's stores (64 where two CTAs each fetch 32-column boxes of an
     // MN-major B); tiles are as wide as TMEM allows and the last one of a row is given to the tensor core at its
     // own, smaller width
