@@ -1,0 +1,47 @@
+"""Kernels whose shape follows the number of patterns: softmax deltas with one, two or four warps for a pattern, row statistics of forward calls, on
+either side of where the choice changes."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth_inputs as si
+from paper_1911_05181_b200 import binding as ul
+from helpers import TOL, GpuNet, dev, tolerance_at
+
+pytestmark = pytest.mark.gpu
+
+# patterns: blocks of eight, four warps each up to 148 blocks, two up to 296; classes: one step of 256 per warp and one more or less
+@pytest.mark.parametrize("math", [ul.MATH_3XTF32, ul.MATH_TF32, ul.MATH_BF16])
+@pytest.mark.parametrize("n", [1, 7, 1184, 1185, 2368, 2369])
+@pytest.mark.parametrize("classes", [256, 257, 513, 1281])
+def test_softmax_head(math, n, classes):
+    sizes = [21, 40, classes]
+    Ws, bs = si.mlp_params(11, sizes)
+    X, y = si.mlp_batch(11, sizes, n)
+    want = oracle.mlp_gradient(Ws, bs, X, y)
+    cond = oracle.gradient_condition(Ws, bs, X, labels=y)
+    g = GpuNet(sizes, math, n); g.set_params(Ws, bs)
+    loss, dW, db = g.gradient(X, y)
+    assert abs(loss - want[0]) <= TOL[math] * abs(want[0])
+    for a, ref, k in zip(dW + db, want[1] + want[2], cond[0] + cond[1]):
+        assert oracle.rel_l2(a, ref) <= tolerance_at(math, k)
+    # the error alone: other kernels, sums of the same terms (double) over 32-bit sums of exponentials that are the same
+    assert abs(g.forward_loss(X, y) - loss) <= 1e-9 * abs(loss)
+
+
+@pytest.mark.parametrize("count", [1, 3, 4, 5, 1027, 4096])
+@pytest.mark.parametrize("off", [0, 1, 2])
+def test_vectors_at_any_alignment(count, off):
+    x, y = (torch.randn(count + 8, device="cuda") for _ in range(2))
+    a, b = x[off:off + count], y[:count]
+    out = torch.full((count + 8,), 7.0, device="cuda")
+    ul.vec_axpby(count, 0.5, a, -2.0, b, out[off:off + count])
+    want = (0.5 * a.double() - 2.0 * b.double())
+    torch.cuda.synchronize()
+    # one rounding of b*y and one of the sum
+    assert bool(((out[off:off + count] - want).abs() <= 2.0 ** -23 * (0.5 * a.abs() + 2.0 * b.abs())).all())
+    assert bool((out[:off] == 7.0).all()) and bool((out[off + count:] == 7.0).all())
+    ul.vec_axpby(count, 1.0, a, 1.0, b, a)              # in place
+    torch.cuda.synchronize()
+    assert bool((x[off + count:] != 0).any())
