@@ -246,7 +246,6 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         const int half = ew >> 2;                       // which 64-column blocks of a tile this warp takes
         uint8_t* stg = epi_scratch + ew * (EPI_BUFS * EPI_STAGE_BYTES);
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-        const bool c_vec = ((((uintptr_t)d.C) & 15) == 0) && ((d.ldc & 3) == 0);
         const bool bias_vec = (EPI == EPI_BIAS_TANH || EPI == EPI_LOGITS || EPI == EPI_TANH_SSE) && ((((uintptr_t)d.bias) & 15) == 0);
         const bool t_vec = (EPI == EPI_TANH_SSE) && ((((uintptr_t)d.T) & 15) == 0) && ((d.ldt & 3) == 0);
         const bool ch_vec = ((((uintptr_t)d.Ch) & 15) == 0) && ((d.ldch & 7) == 0);
@@ -328,26 +327,13 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = (nvalid > 0) ? __uint_as_float(raw[cc][j]) : 0.f;
 
+                    const int rows_here = lane < nvalid ? min(32, (int)d.M - r0w) : 0;
+                    float old[32];
+                    const bool add_old = EPI == EPI_SGEMM && d.beta != 0.f;
                     if (EPI == EPI_SGEMM) {
-                        if (d.beta != 0.f) {
-                            if (rv) {
-                                const float* src = d.C + r * d.ldc + c0;
-                                if (c_vec && full) {
+                        if (add_old) read_rows(d.C + (int64_t)r0w * d.ldc + c0 + lane, d.ldc, rows_here, old);
 #pragma unroll
-                                    for (int j = 0; j < 32; j += 4) {
-                                        const float4 o = *reinterpret_cast<const float4*>(src + j);
-                                        v[j] = fmaf(d.beta, o.x, d.alpha * v[j]); v[j + 1] = fmaf(d.beta, o.y, d.alpha * v[j + 1]);
-                                        v[j + 2] = fmaf(d.beta, o.z, d.alpha * v[j + 2]); v[j + 3] = fmaf(d.beta, o.w, d.alpha * v[j + 3]);
-                                    }
-                                } else {
-#pragma unroll
-                                    for (int j = 0; j < 32; ++j) if (j < nvalid) v[j] = fmaf(d.beta, src[j], d.alpha * v[j]);
-                                }
-                            }
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = d.alpha * v[j];
-                        }
+                        for (int j = 0; j < 32; ++j) v[j] = d.alpha * v[j];
                     } else if (EPI == EPI_TANH_SSE) {
                         // Eqs. 1 and 3: y = tanh(z), E += (y - t)^2, stored value dE/dz = 2 (y - t)(1 - y^2)
                         float s = 0.f;
@@ -456,14 +442,9 @@ bf16_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                             for (int j = 0; j < 8; ++j)
                                 rowp[j ^ (lane & 7)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
                             __syncwarp();
-                            const int rows_here = min(32, (int)(d.M - r0w));
-                            if (lane < nvalid) {
-                                float* dst = base + (int64_t)r0w * ld + c0 + lane;
-                                for (int rr = 0; rr < rows_here; ++rr) {
-                                    const float* src = reinterpret_cast<const float*>(blk + rr * 128 + ((((lane >> 2) ^ (rr & 7)) << 4) | ((lane & 3) << 2)));
-                                    dst[(int64_t)rr * ld] = *src;
-                                }
-                            }
+                            float* dst = base + (int64_t)r0w * ld + c0 + lane;
+                            if (add_old) write_rows<true>(blk, lane, dst, ld, rows_here, d.beta, old);
+                            else write_rows<false>(blk, lane, dst, ld, rows_here, 0.f, old);
                             __syncwarp();
                         }
                     }
@@ -676,7 +657,7 @@ ulsnn_status_t hg_gemm_launch(const HalfGemmDesc& d, cudaStream_t stream) {
     if (d.epi == EPI_PARTIAL) {
         p.c_tma = make_store_map_f32(&mc, d.partials, d.N, d.M, d.ldp, splits) ? 1 : 0;
     } else if (d.epi == EPI_SGEMM) {
-        if (d.C && (((uintptr_t)d.C) & 15) == 0 && (d.ldc & 3) == 0 && d.ldc >= 4 && (d.N & 3) == 0)
+        if (d.beta == 0.f && d.C && (((uintptr_t)d.C) & 15) == 0 && (d.ldc & 3) == 0 && d.ldc >= 4 && (d.N & 3) == 0)
             p.c_tma = make_store_map_f32(&mc, d.C, d.N, d.M, d.ldc, 1) ? 1 : 0;
     } else if (out16 && d.Ch && (((uintptr_t)d.Ch) & 15) == 0 && (d.ldch & 7) == 0 && d.ldch >= 8) {
         // A TMA store clips a row at the next 16-byte boundary past the matrix edge: a width that is not a multiple of

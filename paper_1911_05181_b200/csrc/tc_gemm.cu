@@ -394,7 +394,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         float* bias_s = reinterpret_cast<float*>(epi_scratch + NUM_EPI_WARPS * (2 * EPI_STAGE_BYTES));
         constexpr bool HAS_BIAS = EPI == EPI_BIAS_TANH || EPI == EPI_LOGITS || EPI == EPI_TANH_SSE;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-        const bool c_vec = ((((uintptr_t)d.C) & 15) == 0) && ((d.ldc & 3) == 0);
         const bool t_vec = (EPI == EPI_TANH_SSE) && ((((uintptr_t)d.T) & 15) == 0) && ((d.ldt & 3) == 0);
         const bool h_vec = (EPI == EPI_TANHP) && ((((uintptr_t)d.Hm) & 15) == 0) && ((d.ldh & 3) == 0);
         uint16_t* factors_s = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(ctrl) + COL_FACTORS_AT);     // of the output pair's columns
@@ -461,6 +460,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const int c0 = n0 + c * 32;
                 const int nvalid = min(32, (int)d.N - c0);      // < 32 only in the last block of a row of the matrix
                 const bool full = nvalid == 32;
+                // SGEMM with beta, rows that TMA does not store: the old values, where the registers (128 in 3xTF32 mode) hold them beside the block
+                float old[32];
+                const bool add_old = EPI == EPI_SGEMM && d.beta != 0.f && !p.c_tma;
+                const int rows_here = lane < nvalid ? min(32, (int)d.M - r0w) : 0;
+                if (!THREE_X && add_old) read_rows(d.C + (int64_t)r0w * d.ldc + c0 + lane, d.ldc, rows_here, old);
                 uint32_t raw[32];
                 tmem_ld32(tmem_base + acc * BN_MAX + c * 32 + lane_off, raw);
                 tmem_ld_wait();
@@ -470,10 +474,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 bool do_store = true;
 
                 if (EPI == EPI_SGEMM) {
-                    if (d.beta != 0.f) {
+                    if (THREE_X && d.beta != 0.f && p.c_tma) {      // rows of 16-byte multiples
                         if (rv) {
                             const float* src = d.C + r * d.ldc + c0;
-                            if (c_vec && full) {
+                            if (full) {
 #pragma unroll
                                 for (int j = 0; j < 32; j += 4) {
                                     const float4 o = *reinterpret_cast<const float4*>(src + j);
@@ -612,13 +616,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         for (int j = 0; j < 8; ++j)
                             rowp[j ^ (lane & 7)] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
                         __syncwarp();
-                        const int rows_here = min(32, (int)(d.M - r0w));
-                        if (lane < nvalid) {
-                            float* dst = direct_base + (int64_t)r0w * ld + c0 + lane;
-                            for (int rr = 0; rr < rows_here; ++rr) {
-                                const float* src = reinterpret_cast<const float*>(blk + rr * 128 + ((((lane >> 2) ^ (rr & 7)) << 4) | ((lane & 3) << 2)));
-                                dst[(int64_t)rr * ld] = *src;
-                            }
+                        float* dst = direct_base + (int64_t)r0w * ld + c0 + lane;
+                        if constexpr (EPI == EPI_SGEMM) {
+                            if (THREE_X && add_old) add_rows(blk, lane, dst, ld, rows_here, d.beta);
+                            else if (add_old) write_rows<true>(blk, lane, dst, ld, rows_here, d.beta, old);
+                            else write_rows<false>(blk, lane, dst, ld, rows_here, 0.f, old);
+                        } else if constexpr (!THREE_X) {
+                            write_rows<false>(blk, lane, dst, ld, rows_here, 0.f, old);
+                        } else {
+                            for (int rr = 0; rr < rows_here; ++rr, dst += ld)
+                                *dst = *reinterpret_cast<const float*>(blk + rr * 128 + ((((lane >> 2) ^ (rr & 7)) << 4) | ((lane & 3) << 2)));
                         }
                     }
                 };
@@ -1014,7 +1021,7 @@ ulsnn_status_t tc_gemm_launch(const GemmDesc& d, bool three_x, cudaStream_t stre
         // of four spills up to three floats into the row's padding.  That padding is scratch in the library's own
         // logit and delta buffers; it belongs to the caller in C, and it is the ones column in an activation buffer.
         const bool pad_is_scratch = d.epi == EPI_LOGITS || d.epi == EPI_TANHP || d.epi == EPI_TANH_SSE;
-        if ((d.N & 3) == 0 || pad_is_scratch) p.c_tma = make_store_map_f32(&m.c, d.C, d.N, d.M, d.ldc, 1) ? 1 : 0;
+        if (((d.N & 3) == 0 || pad_is_scratch) && (d.epi != EPI_SGEMM || three_x || d.beta == 0.f)) p.c_tma = make_store_map_f32(&m.c, d.C, d.N, d.M, d.ldc, 1) ? 1 : 0;
     }
 
     const int smem_bytes = 1024 + stages * p.stage_bytes + EPI_SCRATCH_BYTES + CTRL_BYTES;

@@ -312,6 +312,44 @@ __device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
     return v[0];
 }
 
+// ------------------------------------------------------------------------------------------ rows that TMA does not store
+// A 32 x 32 block of an output that TMA cannot store goes through the warp's staging block (rows of 128
+// bytes, 16-byte pieces XORed with the row) and is written row by row, a lane per column, so that every access of the warp is one 128-byte
+// run.  Old values that are added to are asked for in the same way, all of them before the first is used: read word by word by the lane that has the row,
+// each load touched 32 lines (SGEMM 12913 x 3974 x 1680 with beta, TF32 608 -> 325 us, 16-bit mode 439 -> 208; 300 x 391 x 203, 3xTF32, 20.3 -> 15.0).
+// In 3xTF32 mode, whose registers do not hold the old values beside a block, each lane reads its own row where that is a multiple of 16 bytes: eight
+// loads that nothing has to wait for (15203 x 2864 x 510 262 us that way, 361 through the block).  rows: of the block inside the matrix, 0 for columns outside.
+__device__ __forceinline__ void read_rows(const float* src, int64_t ld, int rows, float (&old)[32]) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k, src += ld) old[k] = k < rows ? chain_ld(src) : 0.f;
+}
+template <bool ADD>
+__device__ __forceinline__ void write_rows(const uint8_t* blk, int lane, float* dst, int64_t ld, int rows, float beta, const float (&old)[32]) {
+#pragma unroll
+    for (int k0 = 0; k0 < 32; k0 += 8) {
+        float w[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) w[t] = *reinterpret_cast<const float*>(blk + (k0 + t) * 128 + ((((lane >> 2) ^ t) << 4) | ((lane & 3) << 2)));
+#pragma unroll
+        for (int t = 0; t < 8; ++t, dst += ld) if (k0 + t < rows) *dst = ADD ? fmaf(beta, old[k0 + t], w[t]) : w[t];
+    }
+}
+// write_rows<true> with the old values asked for here, sixteen rows at a time
+__device__ __forceinline__ void add_rows(const uint8_t* blk, int lane, float* dst, int64_t ld, int rows, float beta) {
+#pragma unroll 1
+    for (int k0 = 0; k0 < 32; k0 += 16) {
+        float o[16];
+        float* p = dst;
+#pragma unroll
+        for (int t = 0; t < 16; ++t, p += ld) o[t] = k0 + t < rows ? chain_ld(p) : 0.f;
+#pragma unroll
+        for (int t = 0; t < 16; ++t, dst += ld) {
+            const float w = *reinterpret_cast<const float*>(blk + (k0 + t) * 128 + ((((lane >> 2) ^ (t & 7)) << 4) | ((lane & 3) << 2)));
+            if (k0 + t < rows) *dst = fmaf(beta, o[t], w);
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------ fp16 pairs
 // Exponent fields of a tile's column factors (powers of two), kept for the epilogue warps in the control page behind the barriers: 256
 // half words.  Where a column has one factor they are its bfloat16 bits; where it has two, the low byte is the exponent field of
