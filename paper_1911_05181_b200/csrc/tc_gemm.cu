@@ -934,9 +934,9 @@ ulsnn_status_t launch_mode(bool three_x, int cg, const Maps& m, const TcParams& 
 
 }  // namespace
 
-// Products with more than one 128-row tile are computed by pairs of CTAs (256-row tiles, tcgen05 cta_group::2):
+// Most products with more than one 128-row tile (see cta_pairs) are computed by pairs of CTAs (256-row tiles, tcgen05 cta_group::2):
 // per product instruction each SM then reads half as much of B from its shared memory.
-int tc_cta_group(const GemmDesc& d) { return cta_pairs(d.M, d.N, d.epi) ? 2 : 1; }
+int tc_cta_group(const GemmDesc& d) { return cta_pairs(d.M, d.N, d.epi, d.ctas) ? 2 : 1; }
 int tc_tile_m(const GemmDesc& d) { return BM * tc_cta_group(d); }
 int tc_slots(const GemmDesc& d) { return NUM_SMS / tc_cta_group(d); }
 int tc_colsum_groups() { return 4; }

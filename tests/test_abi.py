@@ -84,6 +84,45 @@ def test_workspace_queries_are_host_only():
         ul.mlp_workspace_bytes([4, 3], 9, 16)
 
 
+def test_three_row_tiles_ask_for_no_more_scratch_than_pairs_of_ctas():
+    """Products of 257-384 rows may run on single CTAs of 128 rows; their slices are those of 256-row tiles on 74 CTA pairs, or fewer: what
+    fitted ulsnn_sgemm_noalloc's array, or needed no workspace at all, still does."""
+    up = lambda x, g: -(-x // g) * g
+    limit = ul.sgemm_noalloc_max_scratch_bytes()
+
+    def pairs(M, N, K, tb):         # slices of a product with two row tiles of 256 rows and 74 pairs to work on them
+        size = M * up(N, 4) * 4
+        tiles = 2 * -(-N // min(256, up(N, 32 if tb == "T" else 64)))
+        least = -(-K // 4096) if K > 8192 else 1
+        s = max(least, max(1, min(-(-2 * 74 // tiles), K // 512)) if tiles < 74 and K >= 1024 else 1)
+        s = -(-K // up(-(-K // s), 32))
+        if s <= 1 or s * size <= limit:
+            return s
+        best, cost, s = 0, 1e300, least         # by estimated time
+        stages = -(-K // 32)
+        while s == least or ((s <= least + 8 or s * tiles <= 2 * 74) and 2 * s <= stages):
+            per = -(-stages // s)
+            used = -(-stages // per)
+            c = -(-used * tiles // 74) * (per + 4) + used * (M * N * 8.0 / 5e6 + 0.15)
+            if (used == s or s == least) and c < cost:
+                best, cost = used, c
+            s += 1
+        return best
+
+    fitted = 0
+    for M in (257, 260, 300, 320, 384):
+        for N in (40, 64, 168, 300, 391, 1000, 3000, 9000, 12544, 12545, 20000):
+            for K in (40, 1023, 1024, 2049, 4000, 16384, 32768, 65536, 131072):
+                for ta, tb in ("NN", "NT", "TN", "TT"):
+                    s = pairs(M, N, K, tb)
+                    most = up(s * M * up(N, 4) * 4, 256) if s > 1 else 0
+                    fitted += 0 < most <= limit
+                    for math in (ul.MATH_3XTF32, ul.MATH_TF32):
+                        got = ul.sgemm_workspace_bytes(ta, tb, M, N, K, math)
+                        assert got <= max(most, ul.sgemm_workspace_bytes(ta, tb, M, N, K, ul.MATH_FP32_SIMT)), (M, N, K, ta, tb, math)
+    assert fitted > 300
+
+
 def test_mlp_create_rejects_bad_workspace():
     lib = ul.lib()
     arr = (ctypes.c_int32 * 3)(8, 4, 2)
