@@ -30,6 +30,20 @@ def test_softmax_head(math, n, classes):
     assert abs(g.forward_loss(X, y) - loss) <= 1e-9 * abs(loss)
 
 
+# a run of 1,024 patterns adds them up sixteen at a time
+@pytest.mark.parametrize("math", [ul.MATH_3XTF32, ul.MATH_TF32, ul.MATH_FP32_SIMT])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 1023, 1024, 1025, 1041])
+def test_bias_gradient_without_a_hidden_layer(math, n):
+    sizes = [21, 131]
+    Ws, bs = si.mlp_params(12, sizes)
+    X, y = si.mlp_batch(12, sizes, n)
+    want = oracle.mlp_gradient(Ws, bs, X, y)
+    cond = oracle.gradient_condition(Ws, bs, X, labels=y)
+    g = GpuNet(sizes, math, n); g.set_params(Ws, bs)
+    _, _, db = g.gradient(X, y)
+    assert oracle.rel_l2(db[0], want[2][0]) <= tolerance_at(math, cond[1][0])
+
+
 @pytest.mark.parametrize("count", [1, 3, 4, 5, 1027, 4096])
 @pytest.mark.parametrize("off", [0, 1, 2])
 def test_vectors_at_any_alignment(count, off):
