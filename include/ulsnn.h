@@ -119,7 +119,7 @@ ulsnn_status_t ulsnn_sgemm_workspace_bytes_for(char transA, char transB, int64_t
  * whose memory budget is fixed up front, under a host framework that owns every allocation, in a callback that
  * must not synchronise the device) cannot size and pass the workspace ulsnn_sgemm_ex wants, and cannot accept
  * the allocate-on-first-need of ulsnn_sgemm.  ulsnn_sgemm_noalloc computes the same product as ulsnn_sgemm_ex with
- * the same `math`, but takes its split-K scratch from a fixed array of ulsnn_sgemm_noalloc_max_scratch_bytes()
+ * the same `math` (never from fp16 pairs: where ulsnn_sgemm_ex takes these, the last bits differ), but takes its split-K scratch from a fixed array of ulsnn_sgemm_noalloc_max_scratch_bytes()
  * (8 MiB) that is part of the library's image on every GPU that loads it.  It calls neither cudaMalloc nor
  * cudaFree nor any allocating routine.
  *  - A product whose scratch does not fit is rejected with ULSNN_ERR_TOO_LARGE and nothing is launched.  What is

@@ -2,8 +2,8 @@
 // the error-compensated 3xTF32 mode (operands as TF32 hi/lo pairs, split on chip, or loaded as a stored pair: B),
 // and the fused epilogues.
 //
-// It computes every product of TF32 mode and of SGEMM, and in 3xTF32 mode those that read the caller's batch (the first and
-// the last of a gradient); the others are fp16-pair products (pair_gemm.cu).
+// It computes every product of TF32 mode, and in 3xTF32 mode those that read the caller's batch (the first and the last of a gradient), those of
+// networks without a hidden layer and SGEMMs that are small or whose operands fp16 pairs do not hold; the others are fp16-pair products (pair_gemm.cu).
 //
 // One persistent CTA per SM, warps with fixed roles (14 warps in 3xTF32 mode, 7 in TF32 mode):
 //   warp 0      TMA producer      global -> swizzled shared-memory stages (cp.async.bulk.tensor, no multicast); in TF32 mode
