@@ -88,8 +88,9 @@ int ulsnn_version(void);
  * values (as much as the operands themselves; left out where that is more than 640 MiB beyond what the product needs otherwise).  Given
  * that much, ulsnn_sgemm_ex converts them and, on the device, looks whether the pairs hold them: no value that is not finite, and so few
  * values below about 2^-15 of the largest in their row of op(A) or column of op(B) that what these lose is below 2^-22 of the sum of the
- * magnitudes of any entry's terms.  If so the products run on the pairs, 1.2 to 1.8 times as fast in all; if not, on TF32
- * parts as with less workspace, with the same result and 5 to 15 % later (values of very different size along a sum, sums of mostly zeros).
+ * magnitudes of any entry's terms.  If so the products run on the pairs, 1.2 to 2.1 times as fast in all; if not, on TF32
+ * parts as with less workspace, with the same result and 20 to 70 us later (values of very different size along a sum, sums of mostly zeros):
+ * a fifth of the smallest such products' time, 5 % of 480 x 3203 x 65536, 1 % of 8192^3.  A smaller workspace spares that.
  * ulsnn_sgemm's own scratch is shared by all its calls on a device: calls on one device must be ordered with respect
  * to each other (one stream, or events), and any call that needs more scratch than every earlier one may synchronise.
  * ULSNN_MATH_BF16: op(A) and op(B) are first rounded to bfloat16 (round to nearest even) into the workspace, which

@@ -14,6 +14,13 @@
 // both sides, infinities, not-a-numbers) the product is formed from TF32 pairs as before.  Both ways are launched; the
 // verdict stays on the device, and the kernels of the way not taken return at once.
 //
+// Operands that fail should not pay for a conversion that nobody reads (480 x 3203 x 65536: 380 us).  So the first blocks to run leave what they have
+// counted of whole rows, or expect of columns from the sample that these are scaled after, and all blocks stop as soon as the test above cannot be met
+// by that, or a value has been found that decides it.  The verdict is "no" wherever these expectations miss the test, whether or not a
+// block was late enough to stop for it: it depends on the operands alone.  Calls whose operands fail, over the same without the conversion,
+// before and after (half zeros, log-normal, one infinity): 480 x 3203 x 65536 1.35-1.37 / 1.05-1.10, 4096^3 1.16 / 1.06-1.09, 2304^3 1.32 / 1.20-1.23, 16000 x 480 x 3203
+// 1.42 / 1.11-1.12, 8192^3 1.05 / 0.99-1.01; operands that pass 0.92-1.02 of the time before, as the operands' blocks run in turn.
+//
 // Bound by memory: every value is read once and written once as four bytes (rows whose scale needs their own largest value: read
 // twice beyond the first 8192, the second time from L2).  Where the sums run across the stored rows, the scale of a column comes
 // from up to 64 of its rows, spread evenly, with three bits to spare: its largest value over all rows would take a pass of its own.
@@ -26,6 +33,8 @@ namespace {
 constexpr int STRIP = 256;                  // columns of a strip: eight per lane
 constexpr int MOST_ROWS = 512;
 constexpr int SAMPLE = 64;                  // rows
+constexpr int EARLY = 64;                   // blocks that leave the counts of their first rows
+constexpr int RESIDENT = 148 * 3;           // blocks that run from the start
 constexpr uint32_t SPARE_BITS = 2;          // a sampled maximum is scaled to 2^12 .. 2^13 instead of 2^14 .. 2^15
 constexpr float OVER = 65504.f, FAINT_VALUE = 0.125f, LOW_VALUE = 128.f;
 
@@ -40,9 +49,30 @@ struct Params {
     uint32_t* state;                        // OPERAND_PAIR_WORDS words
     int64_t K;
 };
-// words of `state`: the verdict, a ticket, whether a value does not fit, then for each operand that is scaled by its rows the largest
-// counts of faint and of low values, eight words for the parts of a row
-enum : int { VERDICT = 0, TICKET = 1, UNFIT = 2, LARGEST = 3 };
+// words of `state`: the verdict, a ticket, then for each operand that is scaled by its rows the largest counts of faint and of low values,
+// eight words for the parts of a row, for each that is scaled by its columns the same two counts as the sample has them, and whether to go on
+enum : int { VERDICT = 0, TICKET = 1, LARGEST = 2, EXPECTED = 34, OUTLOOK = 38 };
+static_assert(OUTLOOK + 1 == OPERAND_PAIR_WORDS, "words");
+enum : uint32_t { GO_ON = 0, ANY_FAINT_DECIDES = 1, STOP = 2 };     // values of OUTLOOK
+
+// What the counts left so far allow: they only grow, and so does this.
+__device__ uint32_t outlook(const Params& p) {
+    const volatile uint32_t* state = p.state;
+    int64_t faint = 0, low = 0;
+    for (int w = 0; w < 2; ++w) {
+        if (!p.m[w].per_row) { faint += state[EXPECTED + 2 * w]; low += state[EXPECTED + 2 * w + 1]; continue; }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { faint += state[LARGEST + 16 * w + i]; low += state[LARGEST + 16 * w + 8 + i]; }
+    }
+    if (faint > 0 && faint > 2 * (p.K - low)) return STOP;
+    return p.K <= low ? ANY_FAINT_DECIDES : GO_ON;
+}
+__device__ void look_out(const Params& p) {        // by one thread, after its block's counts
+    __threadfence();
+    const uint32_t o = outlook(p);
+    if (o != GO_ON) atomicMax(p.state + OUTLOOK, o);
+}
+__device__ __forceinline__ uint32_t current_outlook(const Params& p) { return *(const volatile uint32_t*)(p.state + OUTLOOK); }
 
 // Everything that the conversion counts in set to 0
 __global__ void __launch_bounds__(256) operand_start_kernel(const Params p) {
@@ -75,13 +105,25 @@ __device__ __forceinline__ void store8(__half* dst, int64_t plane, const float (
 // sum, over its G parts, of the largest count of any row's such part.
 template <int G>
 __device__ void convert_rows(const Params& p, const OperandPair& m, int which, int block) {
-    __shared__ uint32_t red[2][8], counts[2][8];
+    __shared__ uint32_t red[2][8], counts[2][8], seen[2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
     const bool vec = (((uintptr_t)m.src) & 15) == 0 && (m.lds & 3) == 0;
     constexpr int HELD = 4;
     uint32_t faint_most = 0, low_most = 0, unfit = 0, turn = 0;
     const int64_t step = (int64_t)p.blocks[which] * (8 / G);
+    auto leave_counts = [&] {           // a word per part, operand and count
+        if (lane == 0) { counts[0][warp] = faint_most; counts[1][warp] = low_most; }
+        __syncthreads();
+        if (threadIdx.x < 2 * G) {
+            const int kind = threadIdx.x / G, of = threadIdx.x % G;
+            uint32_t most = 0;
+#pragma unroll
+            for (int w = of; w < 8; w += G) most = max(most, counts[kind][w]);
+            if (most) atomicMax(p.state + LARGEST + 16 * which + 8 * kind + of, most);
+        }
+    };
     for (int64_t r0 = (int64_t)block * (8 / G); r0 < m.rows; r0 += step, turn ^= 1u) {
+        uint32_t go = (G > 1 ? threadIdx.x : lane) == 0 ? current_outlook(p) : 0u;
         const int64_t r = r0 + warp / G;
         const int64_t width = r < m.rows ? (m.cols + 7) / 8 * 8 : 0;
         const float* s = m.src + r * m.lds;
@@ -105,10 +147,15 @@ __device__ void convert_rows(const Params& p, const OperandPair& m, int which, i
         mx = __reduce_max_sync(0xffffffffu, mx);
         if (G > 1) {
             if (lane == 0) red[turn][warp] = mx;
+            if (threadIdx.x == 0) seen[turn] = go;
             __syncthreads();
 #pragma unroll
             for (int w = 0; w < G; ++w) mx = max(mx, red[turn][warp / G * G + w]);
+            go = seen[turn];
+        } else {
+            go = __shfl_sync(0xffffffffu, go, 0);
         }
+        if (go == STOP && r0 >= step) break;        // all warps of a block write their first rows: they meet after them
         uint32_t faint = 0, low = 0;
         const float scale = pair_scale(mx);
         auto write = [&](int64_t c0, const float (&x)[8]) {
@@ -134,29 +181,30 @@ __device__ void convert_rows(const Params& p, const OperandPair& m, int which, i
         if (lane == 0 && part == 0 && r < m.rows) m.max_bits[r] = mx;
         faint = __reduce_add_sync(0xffffffffu, faint); low = __reduce_add_sync(0xffffffffu, low);
         if (mx != 0u) { faint_most = max(faint_most, faint); low_most = max(low_most, low); }
-    }
-    unfit = __reduce_or_sync(0xffffffffu, unfit);
-    if (lane == 0) {
-        if (unfit) p.state[UNFIT] = 1u;
-        counts[0][warp] = faint_most; counts[1][warp] = low_most;
+        if (__any_sync(0xffffffffu, unfit != 0u || (go == ANY_FAINT_DECIDES && faint != 0u)) && lane == 0) atomicMax(p.state + OUTLOOK, (uint32_t)STOP);
+        if (block < EARLY && r0 < step) {       // its first rows
+            leave_counts();
+            __syncthreads();
+            if (threadIdx.x == 0) look_out(p);
+        }
     }
     __syncthreads();
-    if (threadIdx.x < 2 * G) {          // a word per part, operand and count
-        const int kind = threadIdx.x / G, of = threadIdx.x % G;
-        uint32_t most = 0;
-#pragma unroll
-        for (int w = of; w < 8; w += G) most = max(most, counts[kind][w]);
-        if (most) atomicMax(p.state + LARGEST + 16 * which + 8 * kind + of, most);
-    }
+    leave_counts();
 }
 
 // Rows that are summed across: a block takes a strip of columns through a run of the rows, a warp every eighth of them.  A lane has eight
 // neighbouring columns where the rows can be read 16 bytes at a time, else every 32nd: eight reads of single values that are neighbours in
 // a lane take 70 cycles of the load unit per KB, and 16 when they are neighbours across the warp.
+struct Strip {
+    uint32_t counts[8][STRIP];              // low values in the lower half, faint ones in the upper; runs are at most MOST_ROWS rows
+    uint32_t any[STRIP];
+    uint32_t exponents[2][8][STRIP];        // of the sampled values, four of a column to a word
+    uint32_t low[8], faint[8], columns[8], told;
+};
 template <bool VEC>
-__device__ void convert_columns(const Params& p, const OperandPair& m, int which, int block) {
-    __shared__ uint32_t counts[8][STRIP];           // low values in the lower half, faint ones in the upper; runs are at most MOST_ROWS rows
-    __shared__ uint32_t any[STRIP];
+__device__ void convert_columns(const Params& p, const OperandPair& m, int which, int block, Strip& strip) {
+    auto& counts = strip.counts;
+    auto& any = strip.any;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int strips = (int)((m.cols + STRIP - 1) / STRIP);
     const int64_t c0 = (int64_t)(block % strips) * STRIP + (VEC ? 8 * lane : lane);
@@ -164,6 +212,7 @@ __device__ void convert_columns(const Params& p, const OperandPair& m, int which
     const int64_t width = (m.cols + 7) / 8 * 8;
     constexpr int APART = VEC ? 1 : 32;             // from one of a lane's columns to the next
     any[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) strip.told = 0u;
     uint32_t count[8] = {0, 0, 0, 0, 0, 0, 0, 0}, unfit = 0, some = 0;
     auto load = [&](int64_t r, float (&x)[8]) {
         const float* s = m.src + r * m.lds + c0;
@@ -178,17 +227,28 @@ __device__ void convert_columns(const Params& p, const OperandPair& m, int which
     {
         const int sample = m.rows < SAMPLE ? (int)m.rows : SAMPLE;
         uint32_t mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (c0 < width) {
 #pragma unroll 1
-            for (int i = warp; i < sample; i += 32) {
+        for (int part = 0; part < 2; ++part) {
+            const int i = warp + 32 * part;
+            uint32_t e[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) e[t] = 0xFEFEFEFEu;        // neither faint nor low: no value
+            if (i < sample) {
                 float x[4][8];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) load((int64_t)((uint64_t)min(i + 8 * k, sample - 1) * p.sample_step[which] >> 16), x[k]);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) mx[t] = finite_max(mx[t], magnitude(x[k][t]));
+                    for (int t = 0; t < 8; ++t) {
+                        const uint32_t a = magnitude(x[k][t]);
+                        mx[t] = finite_max(mx[t], a);
+                        if (i + 8 * k < sample) e[t] = __byte_perm(e[t], a >> 23, k == 0 ? 0x3214 : k == 1 ? 0x3240 : k == 2 ? 0x3410 : 0x4210);
+                    }
             }
+            if (block < strips)
+#pragma unroll
+                for (int t = 0; t < 8; ++t) strip.exponents[part][warp][first + APART * t] = e[t];
         }
 #pragma unroll
         for (int t = 0; t < 8; ++t) counts[warp][first + APART * t] = mx[t];
@@ -196,8 +256,36 @@ __device__ void convert_columns(const Params& p, const OperandPair& m, int which
         uint32_t most = 0;
 #pragma unroll
         for (int w = 0; w < 8; ++w) most = max(most, counts[w][threadIdx.x]);
+        if (block < strips) {       // what to expect of the strip's columns: scaled values are below 2^(e - (most + SPARE_BITS) + 15)
+            uint32_t low = 0, faint = 0;
+            const uint32_t field = (most >> 23) + SPARE_BITS;
+            const uint32_t below_low = 0x01010101u * (field > 7 ? min(field - 7, 253u) : 0u), below_faint = 0x01010101u * (field > 17 ? min(field - 17, 253u) : 0u);
+            if (most)
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) {
+                        const uint32_t e = strip.exponents[part][w][threadIdx.x];
+                        low += __popc(__vcmpltu4(e, below_low)) >> 3;
+                        faint += __popc(__vcmpltu4(e, below_faint) & __vcmpne4(e, 0u)) >> 3;
+                    }
+            const uint32_t columns = __reduce_add_sync(0xffffffffu, most ? 1u : 0u);
+            low = __reduce_add_sync(0xffffffffu, low); faint = __reduce_add_sync(0xffffffffu, faint);
+            if (lane == 0) { strip.low[warp] = low; strip.faint[warp] = faint; strip.columns[warp] = columns; }
+        }
         most = (most ? min((most >> 23) + SPARE_BITS, 254u) : 127u) << 23;      // nothing but zeros seen: as if the largest were 1
         __syncthreads();
+        if (block < strips && threadIdx.x == 0) {
+            uint64_t low = 0, faint = 0, columns = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) { low += strip.low[w]; faint += strip.faint[w]; columns += strip.columns[w]; }
+            if (columns) {
+                const uint64_t of = columns * (uint64_t)sample;
+                if (faint) atomicMax(p.state + EXPECTED + 2 * which, (uint32_t)((uint64_t)m.rows * faint / of));
+                if (low) atomicMax(p.state + EXPECTED + 2 * which + 1, (uint32_t)((uint64_t)m.rows * low / of));
+            }
+            look_out(p);
+        }
         counts[0][threadIdx.x] = most;
         const int64_t c = (int64_t)(block % strips) * STRIP + threadIdx.x;
         if (block < strips && c < m.cols) m.max_bits[c] = most;
@@ -207,43 +295,50 @@ __device__ void convert_columns(const Params& p, const OperandPair& m, int which
 #pragma unroll
     for (int t = 0; t < 8; ++t) scale[t] = pair_scale(counts[0][first + APART * t]);
     __syncthreads();
-    if (c0 < width) {
-        auto write = [&](int64_t r, const float (&x)[8]) {
-            float v[8];
+    auto write = [&](int64_t r, const float (&x)[8]) {
+        float v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            v[t] = x[t] * scale[t];
+            const float a = fabsf(v[t]);
+            const bool nz = magnitude(x[t]) != 0u;
+            unfit |= !(a < OVER) ? 1u : 0u;
+            some |= nz ? 1u << t : 0u;
+            count[t] += (a < LOW_VALUE ? 1u : 0u) + (a < FAINT_VALUE && nz ? 0x10000u : 0u);
+        }
+        __half* dst = m.dst + r * m.ld + c0;
+        if (VEC) {
+            if (c0 < width) store8(dst, m.plane, v);
+        } else {
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-                v[t] = x[t] * scale[t];
-                const float a = fabsf(v[t]);
-                const bool nz = magnitude(x[t]) != 0u;
-                unfit |= !(a < OVER) ? 1u : 0u;
-                some |= nz ? 1u << t : 0u;
-                count[t] += (a < LOW_VALUE ? 1u : 0u) + (a < FAINT_VALUE && nz ? 0x10000u : 0u);
+                if (c0 + 32 * t >= width) break;
+                const __half h = __float2half_rn(v[t]);
+                dst[32 * t] = h;
+                dst[m.plane + 32 * t] = __float2half_rn(v[t] - __half2float(h));
             }
-            __half* dst = m.dst + r * m.ld + c0;
-            if (VEC) store8(dst, m.plane, v);
-            else {
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    if (c0 + 32 * t >= width) break;
-                    const __half h = __float2half_rn(v[t]);
-                    dst[32 * t] = h;
-                    dst[m.plane + 32 * t] = __float2half_rn(v[t] - __half2float(h));
-                }
-            }
-        };
-        constexpr int AHEAD = 4;
-        for (int64_t r = r0 + warp; r < r1; r += 8 * AHEAD) {
-            float x[AHEAD][8];
-#pragma unroll
-            for (int k = 0; k < AHEAD; ++k) if (r + 8 * k < r1) load(r + 8 * k, x[k]);
-#pragma unroll
-            for (int k = 0; k < AHEAD; ++k) if (r + 8 * k < r1) write(r + 8 * k, x[k]);
         }
+    };
+    constexpr int AHEAD = 4;
+    for (int64_t r = r0 + warp; r < r1; r += 8 * AHEAD) {
+        uint32_t go = lane == 0 ? current_outlook(p) : 0u;
+        float x[AHEAD][8];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) if (r + 8 * k < r1) load(r + 8 * k, x[k]);
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) if (r + 8 * k < r1) write(r + 8 * k, x[k]);
+        go = __shfl_sync(0xffffffffu, go, 0);
+        if (go == STOP) break;
+        uint32_t counted = 0;
+        if (go == ANY_FAINT_DECIDES) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) counted |= count[t];
+        }
+        // a value that decides: one warp of the block tells the others
+        if (__any_sync(0xffffffffu, unfit != 0u || counted >> 16 != 0u) && lane == 0 && atomicExch(&strip.told, 1u) == 0u) atomicMax(p.state + OUTLOOK, (uint32_t)STOP);
     }
 #pragma unroll
     for (int t = 0; t < 8; ++t) counts[warp][first + APART * t] = count[t];
-    unfit = __reduce_or_sync(0xffffffffu, unfit);
-    if (lane == 0 && unfit) p.state[UNFIT] = 1u;
     __syncthreads();
 #pragma unroll
     for (int t = 0; t < 8; ++t) if ((some >> t) & 1u) any[first + APART * t] = 1u;
@@ -262,11 +357,22 @@ __device__ void convert_columns(const Params& p, const OperandPair& m, int which
 __global__ void __launch_bounds__(256, 3) operand_pairs_kernel(const Params p) {
     chain_wait();
     __shared__ uint32_t ticket, most[8][2];
-    const int which = (int)blockIdx.x < p.blocks[0] ? 0 : 1, block = (int)blockIdx.x - (which ? p.blocks[0] : 0);
+    __shared__ Strip strip;
+    // the operands' blocks in turn, so that the first of both run early
+    const int in_turn = 2 * min(p.blocks[0], p.blocks[1]), b = (int)blockIdx.x;
+    const int which = b < in_turn ? b & 1 : p.blocks[1] > p.blocks[0] ? 1 : 0, block = b < in_turn ? b >> 1 : b - in_turn / 2;
     const OperandPair& m = p.m[which];
-    if (!m.per_row) {
-        if ((((uintptr_t)m.src) & 15) == 0 && (m.lds & 3) == 0) convert_columns<true>(p, m, which, block);
-        else convert_columns<false>(p, m, which, block);
+    bool stopped = false;
+    if (b >= RESIDENT) {
+        if (threadIdx.x == 0) ticket = current_outlook(p);
+        __syncthreads();
+        stopped = ticket == STOP;
+        __syncthreads();
+    }
+    if (stopped) {
+    } else if (!m.per_row) {
+        if ((((uintptr_t)m.src) & 15) == 0 && (m.lds & 3) == 0) convert_columns<true>(p, m, which, block, strip);
+        else convert_columns<false>(p, m, which, block, strip);
     }
     else if (p.warps_per_row[which] == 8) convert_rows<8>(p, m, which, block);
     else if (p.warps_per_row[which] == 4) convert_rows<4>(p, m, which, block);
@@ -298,7 +404,12 @@ __global__ void __launch_bounds__(256, 3) operand_pairs_kernel(const Params p) {
         for (int i = 0; i < 8; ++i) { f = max(f, most[i][0]); l = max(l, most[i][1]); }
         faint += f; low += l;
     }
-    if (threadIdx.x == 0) p.state[VERDICT] = state[UNFIT] == 0u && (faint == 0 || faint <= 2 * (p.K - low)) ? 1u : 0u;
+    if (threadIdx.x == 0) {
+        // blocks that stopped have left no counts, but then their reason is in what the others left
+        const uint32_t o = max(outlook(p), state[OUTLOOK]);
+        const bool holds = faint == 0 || faint <= 2 * (p.K - low);
+        p.state[VERDICT] = o != STOP && !(o == ANY_FAINT_DECIDES && faint > 0) && holds ? 1u : 0u;
+    }
 }
 
 }  // namespace
