@@ -14,9 +14,10 @@ from helpers import TOL, GpuNet, dev
 pytestmark = pytest.mark.gpu
 
 
+# without events the slices of all layers are added up by one launch up to 32 MB of them, layer by layer beyond (36 MB): the same bits as with events
 @pytest.mark.parametrize("math", [ul.MATH_3XTF32, ul.MATH_TF32, ul.MATH_BF16, ul.MATH_FP32_SIMT])
-def test_layer_events_mark_final_gradients(math):
-    sizes, n = [40, 64, 48, 33], 3000
+@pytest.mark.parametrize("sizes,n", [([40, 64, 48, 33], 3000), ([64, 3000, 3003], 200)])
+def test_layer_events_mark_final_gradients(math, sizes, n):
     Ws, bs = si.mlp_params(9, sizes)
     X, y = si.mlp_batch(9, sizes, n)
     want = oracle.mlp_gradient(Ws, bs, X, y)

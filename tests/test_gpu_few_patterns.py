@@ -56,6 +56,29 @@ def test_vectors_at_any_alignment(count, off):
     # one rounding of b*y and one of the sum
     assert bool(((out[off:off + count] - want).abs() <= 2.0 ** -23 * (0.5 * a.abs() + 2.0 * b.abs())).all())
     assert bool((out[:off] == 7.0).all()) and bool((out[off + count:] == 7.0).all())
-    ul.vec_axpby(count, 1.0, a, 1.0, b, a)              # in place
-    torch.cuda.synchronize()
-    assert bool((x[off + count:] != 0).any())
+    for into in (a, b):                                 # in place: the result, and nothing around it
+        was, sum_ = [t.clone() for t in (x, y)], a.double() + b.double()
+        ul.vec_axpby(count, 1.0, a, 1.0, b, into)
+        torch.cuda.synchronize()
+        assert bool(((into - sum_).abs() <= 2.0 ** -24 * sum_.abs()).all())       # 1*y is exact: one rounding
+        into.copy_((was[0][off:] if into is a else was[1])[:count])
+        assert torch.equal(x, was[0]) and torch.equal(y, was[1])
+
+
+@pytest.mark.parametrize("inputs,units", [(1, 1), (5, 3), (16, 4), (33, 31), (64, 129)])
+@pytest.mark.parametrize("off", [0, 1, 2])
+def test_parameter_step_at_any_alignment(inputs, units, off):
+    net = ul.Mlp([inputs, units], ul.MATH_FP32_SIMT, 4)
+    lr = 0.375
+    flat = [torch.randn(inputs * units + 8, device="cuda"), torch.randn(units + 8, device="cuda")]
+    grads = [torch.randn_like(t) for t in flat]
+    for of_w, of_g in ((off, off), (off, 0), (0, off)):
+        was = [t.clone() for t in flat]
+        counts = (inputs * units, units)
+        w, g = [t[of_w:of_w + c] for t, c in zip(flat, counts)], [t[of_g:of_g + c] for t, c in zip(grads, counts)]
+        net.sgd_step([w[0]], [w[1]], [g[0]], [g[1]], lr)
+        torch.cuda.synchronize()
+        for t, before, d, c in zip(flat, was, g, counts):
+            want = before[of_w:of_w + c].double() - lr * d.double()
+            assert bool(((t[of_w:of_w + c] - want).abs() <= 2.0 ** -24 * want.abs()).all())         # a fused multiply-add rounds once
+            assert torch.equal(t[:of_w], before[:of_w]) and torch.equal(t[of_w + c:], before[of_w + c:])
