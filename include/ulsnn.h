@@ -45,7 +45,8 @@ typedef int ulsnn_status_t;
 typedef enum {
     ULSNN_MATH_3XTF32    = 0,  /* tensor cores, each operand split hi+lo, three products: fp32-level accuracy.  TF32 parts keep 22 bits of
                                   any value.  Large products of ulsnn_sgemm_ex use scaled fp16 parts where a test of the operands shows
-                                  that the sums lose no more by them.  Inside a network the parts are scaled fp16, with scales per unit, class, pattern or row of
+                                  that what these drop of values far below the largest in their row or column is below 2^-25 of the sum of
+                                  the magnitudes of any entry's terms, half of what one fp32 addition may round.  Inside a network the parts are scaled fp16, with scales per unit, class, pattern or row of
                                   the weights: what is below 2^-27 of the largest value (activations: of its bound) in the same row or column
                                   is dropped */
     ULSNN_MATH_TF32      = 1,  /* tensor cores, operands truncated to TF32 (10-bit mantissa): fast mode */
@@ -87,7 +88,7 @@ int ulsnn_version(void);
  * ULSNN_MATH_3XTF32, large products: ulsnn_sgemm_workspace_bytes_for also includes the room for both operands as pairs of scaled fp16
  * values (as much as the operands themselves; left out where that is more than 640 MiB beyond what the product needs otherwise).  Given
  * that much, ulsnn_sgemm_ex converts them and, on the device, looks whether the pairs hold them: no value that is not finite, and so few
- * values below about 2^-15 of the largest in their row of op(A) or column of op(B) that what these lose is below 2^-22 of the sum of the
+ * values below about 2^-15 of the largest in their row of op(A) or column of op(B) that what these lose is below 2^-25 of the sum of the
  * magnitudes of any entry's terms.  If so the products run on the pairs, 1.2 to 2.1 times as fast in all; if not, on TF32
  * parts as with less workspace, with the same result and 20 to 70 us later (values of very different size along a sum, sums of mostly zeros):
  * a fifth of the smallest such products' time, 5 % of 480 x 3203 x 65536, 1 % of 8192^3.  A smaller workspace spares that.

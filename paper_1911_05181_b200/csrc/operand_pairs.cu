@@ -7,10 +7,10 @@
 //     faint   values not 0 with |x'| < 2^-3
 //     low     values with |x'| < 2^7, zeros among them
 // and the product may be formed from the pairs if for the largest counts of both operands (rows and columns without a value do not count)
-//     faint_A + faint_B <= 2 (K - low_A - low_B)   or   faint_A + faint_B = 0,
+//     4 (faint_A + faint_B) <= K - low_A - low_B   or   faint_A + faint_B = 0,
 // and every value is finite and below 65504.  For then, of any entry of the product, what the faint values lose is at most
-// 2^-25 2^16 (faint_A + faint_B), while at least K - low_A - low_B of its terms are 2^14 or more: the loss is below 2^-22 of the sum of the
-// terms' magnitudes, which is the rounding of a pair itself.  Where the test fails (values of very different size along a sum, mostly zeros on
+// 2^-25 2^16 (faint_A + faint_B), while at least K - low_A - low_B of its terms are 2^14 or more: the loss is below 2^-25 of the sum of the
+// terms' magnitudes, an eighth of the rounding of a pair itself and half of what one addition in 32 bits may round.  Where the test fails (values of very different size along a sum, mostly zeros on
 // both sides, infinities, not-a-numbers) the product is formed from TF32 pairs as before.  Both ways are launched; the
 // verdict stays on the device, and the kernels of the way not taken return at once.
 //
@@ -64,7 +64,7 @@ __device__ uint32_t outlook(const Params& p) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) { faint += state[LARGEST + 16 * w + i]; low += state[LARGEST + 16 * w + 8 + i]; }
     }
-    if (faint > 0 && faint > 2 * (p.K - low)) return STOP;
+    if (faint > 0 && 4 * faint > p.K - low) return STOP;
     return p.K <= low ? ANY_FAINT_DECIDES : GO_ON;
 }
 __device__ void look_out(const Params& p) {        // by one thread, after its block's counts
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(256, 3) operand_pairs_kernel(const Params p) {
     if (threadIdx.x == 0) {
         // blocks that stopped have left no counts, but then their reason is in what the others left
         const uint32_t o = max(outlook(p), state[OUTLOOK]);
-        const bool holds = faint == 0 || faint <= 2 * (p.K - low);
+        const bool holds = faint == 0 || 4 * faint <= p.K - low;
         p.state[VERDICT] = o != STOP && !(o == ANY_FAINT_DECIDES && faint > 0) && holds ? 1u : 0u;
     }
 }

@@ -86,6 +86,12 @@ def _spoil(name, A, B):
     if name == "few faint values":              # a loss that the sums' other terms cover
         A[:, 3] *= 1e-9; B[:, 4] *= 1e-12
         return True
+    if name == "every eighth value faint":      # what they lose is about as much as the test lets pass
+        A[:, ::8] *= 2.0 ** -19
+        return True
+    if name == "every fourth value faint":      # and more
+        A[:, ::4] *= 2.0 ** -19
+        return False
     if name == "sizes that cancel":             # what is faint in A meets what is large in B
         A[:, ::2] *= 1e-9; B[1::2] *= 1e-9
         return False
@@ -104,7 +110,8 @@ def _spoil(name, A, B):
     raise ValueError(name)
 
 
-@pytest.mark.parametrize("name", ["zero rows and columns", "tiny and huge", "few faint values", "sizes that cancel", "beyond the sample", "infinity",
+@pytest.mark.parametrize("name", ["zero rows and columns", "tiny and huge", "few faint values", "every eighth value faint",
+                                  "every fourth value faint", "sizes that cancel", "beyond the sample", "infinity",
                                   "not a number", "half zeros on both sides"])
 @pytest.mark.parametrize("ta,tb,M,N,K", [("N", "N", 2304, 2052, 2052), ("T", "T", 2050, 2301, 2047), ("N", "T", 2310, 2305, 2048)])
 def test_what_the_pairs_hold(name, ta, tb, M, N, K):
@@ -120,9 +127,9 @@ def test_what_the_pairs_hold(name, ta, tb, M, N, K):
     b = (dB if tb == "N" else dB.t()).double()
     want, terms = (a @ b).cpu().numpy(), (a.abs() @ b.abs()).cpu().numpy()
     # Error of an entry in units of its own terms: the TF32 pairs' worst, which has the same roundings of pairs and more truncations,
-    # and the 2^-22 that the test of the operands lets faint values lose.  What is below 1e-37 is no normal number.
+    # and the 2^-25 that the test of the operands lets faint values lose.  What is below 1e-37 is no normal number.
     off = lambda x: (np.maximum(np.abs(x - want) - 1e-37, 0) / np.maximum(terms, 1e-300)).max()
-    assert off(got) <= off(plain) + 2.0 ** -22
+    assert off(got) <= off(plain) + 2.0 ** -25
 
 
 # M, N, K of which pairs and TF32 parts take different numbers of slices along K: 2 and 5, 1 and 4, 12 and 13
