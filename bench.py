@@ -51,16 +51,16 @@ NOMINAL_TF32_OVER_BF16 = 0.5        # dense TF32 tensor rate is half the BF16 ra
 # traffic is proportional but for the slices' partial products (a few per cent).  Softmax head; reported only while the library still is
 # the version the counters were taken on; null otherwise.
 NCU_TRAFFIC = {
-    "library_version": 111,
-    ("config3", "3xtf32", (65536, 3203, 480)): 4 * (41.396480e6 + 159.556864e6),
-    ("config3", "3xtf32", (65536, 480, 3203)): 4 * (280.179456e6 + 24.333824e6),
-    ("config3", "3xtf32", (3203, 481, 65536)): 4 * (255.164928e6 + 17.678336e6),
-    ("config3", "tf32", (65536, 3203, 480)): 4 * (40.698880e6 + 157.150720e6),
-    ("config3", "tf32", (65536, 480, 3203)): 4 * (256.758528e6 + 18.550016e6),
-    ("config3", "tf32", (3203, 481, 65536)): 4 * (253.641984e6 + 32.606720e6),
-    ("config3", "bf16", (65536, 3203, 480)): 2 * (39.448832e6 + 168.657152e6),
-    ("config3", "bf16", (65536, 480, 3203)): 2 * (256.808704e6 + 18.214400e6),
-    ("config3", "bf16", (3203, 481, 65536)): 2 * (256.340992e6 + 31.413504e6),
+    "library_version": 112,
+    ("config3", "3xtf32", (65536, 3203, 480)): 4 * (41.391104e6 + 158.628864e6),
+    ("config3", "3xtf32", (65536, 480, 3203)): 4 * (279.368960e6 + 22.989056e6),
+    ("config3", "3xtf32", (3203, 481, 65536)): 4 * (255.163392e6 + 17.976832e6),
+    ("config3", "tf32", (65536, 3203, 480)): 4 * (40.771840e6 + 156.659200e6),
+    ("config3", "tf32", (65536, 480, 3203)): 4 * (256.630016e6 + 17.988352e6),
+    ("config3", "tf32", (3203, 481, 65536)): 4 * (252.879104e6 + 31.049728e6),
+    ("config3", "bf16", (65536, 3203, 480)): 2 * (39.412992e6 + 168.593664e6),
+    ("config3", "bf16", (65536, 480, 3203)): 2 * (255.471872e6 + 18.379264e6),
+    ("config3", "bf16", (3203, 481, 65536)): 2 * (256.293888e6 + 29.253376e6),
 }
 # cuBLAS through torch.matmul, 8192^3, on this machine's B200s (`--workload peaks`): TF32 allowed, best of 10 isolated
 # calls and 4 s back to back under the power cap (SM clock 1042 MHz of 1965).  Printed beside the peak the fractions use.
